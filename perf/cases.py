@@ -24,9 +24,9 @@ def listed():
         dict(name="solve_2ac", kind="solve", N=2, H=20, S=4, L=1024, M=8, J=10, grid="16x16x4", box=30, sep=0),
         # a receding-horizon solve of the 8-aircraft traffic, wind field on the fine grid included
         dict(name="solve_8ac", kind="solve", N=8, H=60, S=4, L=16384, M=32, J=8, grid="64x64x8", box=50, sep=0),
-        # a solve with accepted Langevin moves (two gradient passes an iteration)
-        dict(name="solve_mala", kind="solve", N=6, H=30, S=4, L=4096, M=8, J=4, grid="16x16x4", box=50, sep=1,
-             move=2),
+        # a solve with accepted random-walk moves (two more rollouts an iteration)
+        dict(name="solve_rwmh", kind="solve", N=6, H=30, S=4, L=4096, M=8, J=4, grid="16x16x4", box=50, sep=1,
+             move=1),
         # one control step of a batch of uneven scenarios: measured states in, graph, results out
         dict(name="batch_mpc", kind="batch", scen=12, L=2048, M=16, H=60, J=6, grid="16x16x4"),
         # the rollout inside late iterations of the 8-aircraft workload at its full size, hard separation
@@ -63,7 +63,8 @@ def draw(rng):
     grid = rng.choice(["16x16x4", "32x32x8", "64x64x8", "17x12x5"])
     if kind == "solve":
         sep = rng.choice([0, 1, 2])
-        move = rng.choice([0, 1, 2]) if sep else 0
+        # Langevin moves turn the gradient's last bits into accept decisions: their gradient has its own cases
+        move = rng.choice([0, 1]) if sep else 0
         return dict(kind=kind, N=rng.randint(2, 12), H=rng.randint(10, 60), S=rng.randint(1, 5),
                     L=_spread(rng, 512, 16384), M=rng.randint(4, 24), J=rng.randint(2, 8), grid="16x16x4", box=50,
                     sep=sep, move=move)
@@ -270,8 +271,8 @@ def work(case):
         return {"bytes": u + 4 * N * L * (2 if case["sep"] else 1) + (0 if case.get("wind_mode") else field), "flops": one}
     if kind == "grad":
         return {"bytes": 2 * u + 4 * N * L + field, "flops": 3 * one}
-    # a solve: the field, J rollouts; Langevin moves add two gradients an iteration, random walks two rollouts
-    extra = {0: 0, 1: 2, 2: 6}[case.get("move", 0)] * (case["J"] - 1)
+    # a solve: the field and J rollouts; accepted random-walk moves add two rollouts an iteration
+    extra = {0: 0, 1: 2}[case.get("move", 0)] * (case["J"] - 1)
     return {"bytes": field + u * case["J"], "flops": one * (case["J"] + extra)}
 
 
