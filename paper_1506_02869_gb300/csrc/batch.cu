@@ -21,6 +21,7 @@
 #include <algorithm>
 
 #include "rollout_tile.cuh"
+#include "wind_normals.cuh"
 
 namespace tma {
 
@@ -204,55 +205,22 @@ __global__ void __launch_bounds__(256) batch_init(const BatchScen *__restrict__ 
 // As the single-scenario kernel, over (scenario of the group, sample, node);
 // every scenario keys its own normals and uses its own MPC step.  w.M is the
 // group's sample count (scenarios x M_scen).
+template <int LANES>
 __global__ void __launch_bounds__(128) batch_wind_normals_ar(const WindC w, int s0, int M_scen,
                                                              const BatchScen *__restrict__ scen,
                                                              const DynState *__restrict__ dyns,
                                                              float *__restrict__ Btmp)
 {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)w.M * w.nxy) return;
-    const int ms = (int)(t / w.nxy);           // (scenario in group, sample) < w.M
-    const int q = (int)(t - (long long)ms * w.nxy);
+    const long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+    const int iz = threadIdx.x % LANES;
+    const bool on = t < (long long)w.M * w.nxy && iz < w.nz;
+    const long long tc = min(t, (long long)w.M * w.nxy - 1);
+    const int ms = (int)(tc / w.nxy);          // (scenario in group, sample) < w.M
+    const int q = (int)(tc - (long long)ms * w.nxy);
     const int sl = ms / M_scen, m = ms - sl * M_scen;
     const int s = s0 + sl;
-    const uint32_t mpc = dyns[s].mpc_step;
-    const uint32_t k0 = scen[s].key0, k1 = scen[s].key1;
-    const int nz = w.nz;
-    float B[2][TMA_MAX_GRID_Z];
-#pragma unroll
-    for (int iz = 0; iz < TMA_MAX_GRID_Z; ++iz) B[0][iz] = B[1][iz] = 0.0f;
-    float *row = Btmp + (size_t)q * w.ldb;
-    for (int k = 0; k < w.H; ++k) {
-#pragma unroll
-        for (int iz = 0; iz < TMA_MAX_GRID_Z; ++iz) {
-            if (iz < nz) {
-                const uint4 r = draw(k0, k1, (uint32_t)(q * nz + iz), (uint32_t)m << 8, (uint32_t)k, 3u, 0u, mpc);
-                const float2 n = box_muller(r.x, r.y);
-                if (k == 0) {
-                    B[0][iz] = n.x;
-                    B[1][iz] = n.y;
-                } else {
-                    B[0][iz] = fmaf(w.a, B[0][iz], w.b * n.x);
-                    B[1][iz] = fmaf(w.a, B[1][iz], w.b * n.y);
-                }
-            }
-        }
-        float *o = row + ((size_t)ms * w.H + k) * (size_t)(2 * nz);
-#pragma unroll
-        for (int iz = 0; iz < TMA_MAX_GRID_Z; ++iz) {
-            if (iz < nz) {
-                float ax = 0.0f, ay = 0.0f;
-#pragma unroll
-                for (int jz = 0; jz <= iz; ++jz) {
-                    const float lz = w.Lz[iz * TMA_MAX_GRID_Z + jz];
-                    ax = fmaf(lz, B[0][jz], ax);
-                    ay = fmaf(lz, B[1][jz], ay);
-                }
-                o[2 * iz] = ax;
-                o[2 * iz + 1] = ay;
-            }
-        }
-    }
+    wind_normals_column<LANES>(w, scen[s].key0, scen[s].key1, 3u, dyns[s].mpc_step, m, q, iz, on,
+                               Btmp + (size_t)q * w.ldb + (size_t)ms * w.H * (size_t)(2 * w.nz));
 }
 
 // --------------------------------------------------------------- selection
@@ -515,7 +483,14 @@ cudaError_t launch_batch_init(const BatchScen *scen, const int *seg_scen, const 
 cudaError_t launch_batch_wind_normals(const WindC &w, int s0, int M_scen, const BatchScen *scen,
                                       const DynState *dyns, float *Btmp, cudaStream_t st)
 {
-    batch_wind_normals_ar<<<blocks_for((long long)w.M * w.nxy, 128), 128, 0, st>>>(w, s0, M_scen, scen, dyns, Btmp);
+    const int lanes = wind_column_lanes(w.nz);
+    const unsigned grid = blocks_for((long long)w.M * w.nxy * lanes, 128);
+    switch (lanes) {
+    case 2: batch_wind_normals_ar<2><<<grid, 128, 0, st>>>(w, s0, M_scen, scen, dyns, Btmp); break;
+    case 4: batch_wind_normals_ar<4><<<grid, 128, 0, st>>>(w, s0, M_scen, scen, dyns, Btmp); break;
+    case 8: batch_wind_normals_ar<8><<<grid, 128, 0, st>>>(w, s0, M_scen, scen, dyns, Btmp); break;
+    default: batch_wind_normals_ar<16><<<grid, 128, 0, st>>>(w, s0, M_scen, scen, dyns, Btmp); break;
+    }
     count_launch();
     return cudaGetLastError();
 }

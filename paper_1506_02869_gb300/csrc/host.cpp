@@ -105,7 +105,7 @@ bool cholesky_lower(std::vector<double> &A, int n)
     return true;
 }
 
-// Horizontal factor L_xy (FP32, zero-padded) cached per grid and rate.
+// Horizontal factor L_xy (FP32, transposed, zero-padded) cached per grid and rate.
 struct LxyEntry {
     std::vector<float> L;
     int lda;
@@ -138,7 +138,7 @@ static std::shared_ptr<LxyEntry> horizontal_factor(const tma_problem &p)
     e->lda = ((n + 127) / 128) * 128;
     e->L.assign((size_t)e->lda * e->lda, 0.0f);
     for (int a = 0; a < n; ++a)
-        for (int b = 0; b <= a; ++b) e->L[(size_t)a * e->lda + b] = (float)R[(size_t)a * n + b];
+        for (int b = 0; b <= a; ++b) e->L[(size_t)b * e->lda + a] = (float)R[(size_t)a * n + b];
     std::lock_guard<std::mutex> g(g_lxy_mu);
     g_lxy[key] = e;
     return e;
@@ -224,7 +224,10 @@ static ProblemC derive_problem(const tma_problem &p, const tma_aircraft *aircraf
     P.S = p.S;
     P.M = p.M;
     P.G = next_pow2(p.N);
-    P.P = p.grid[0] * p.grid[1] * p.grid[2];
+    const WindLayout wl = wind_layout(p.grid[0], p.grid[1], p.grid[2]);
+    P.P = wl.P;
+    P.pitch = wl.pitch;
+    P.plane = wl.plane;
     for (int d = 0; d < 3; ++d) {
         P.grid[d] = p.grid[d];
         P.box_lo[d] = (float)p.box_lo[d];
@@ -560,7 +563,8 @@ tma_status tma_create(const tma_problem *prob, const tma_aircraft *aircraft, tma
         const size_t L = (size_t)p.L, N = (size_t)p.N, M = (size_t)p.M, H = (size_t)p.H;
         const int nx = p.grid[0], ny = p.grid[1], nz = p.grid[2];
         const int nxy = nx * ny;
-        const size_t P = (size_t)nxy * nz;
+        const WindLayout wl = wind_layout(nx, ny, nz);
+        const size_t P = (size_t)wl.P;
         auto fail = [&](cudaError_t e) {
             free_all(s);
             delete s;
@@ -599,6 +603,8 @@ tma_status tma_create(const tma_problem *prob, const tma_aircraft *aircraft, tma
         w.M = p.M;
         w.H = p.H;
         w.nxy = nxy;
+        w.ny = ny;
+        w.out = wl;
         w.nz = nz;
         w.ncol = (int)(M * H * 2 * nz);
         w.ldb = ((w.ncol + 127) / 128) * 128;
@@ -778,7 +784,7 @@ tma_status tma_set_state(tma_solver *s, const tma_state *h_x0, uint32_t mpc_step
     return TMA_OK;
 }
 
-static tma_status gen_wind(tma_solver *s, cudaStream_t st);
+static tma_status gen_wind(tma_solver *s, cudaStream_t st, float *d_W = nullptr);
 
 // Choose the rollout kernel's launch-bound variant by timing every valid
 // candidate on this solver's workload (uniform initial controls, at most 8192
@@ -836,11 +842,11 @@ static tma_status autotune_rollout(tma_solver *s)
     return r;
 }
 
-static tma_status gen_wind(tma_solver *s, cudaStream_t st)
+static tma_status gen_wind(tma_solver *s, cudaStream_t st, float *d_W)
 {
     StageTimer t(s, 0, st);
     TMA_CUDA(launch_wind_normals_ar(s->wind, s->d_dyn, s->d_Btmp, st));
-    TMA_CUDA(launch_wind_gemm(s->wind, s->d_Lxy, s->lda, s->d_Btmp, s->d_W, st));
+    TMA_CUDA(launch_wind_gemm(s->wind, s->d_Lxy, s->lda, s->d_Btmp, s->d_W, st, d_W));
     s->wind_ready = true;
     return TMA_OK;
 }
@@ -849,14 +855,7 @@ tma_status tma_wind_field(tma_solver *s, float *d_W, tma_stream_t stream)
 {
     if (!s) return TMA_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    tma_status r = gen_wind(s, st);
-    if (r != TMA_OK) return r;
-    if (d_W) {
-        // the solver keeps float4 (own value, value one level up) per node; copy the own values
-        const size_t rows = (size_t)s->prob.M * s->prob.H * s->P.P;
-        TMA_CUDA(cudaMemcpy2DAsync(d_W, 8, s->d_W, 16, 8, rows, cudaMemcpyDeviceToDevice, st));
-    }
-    return TMA_OK;
+    return gen_wind(s, st, d_W);
 }
 
 static tma_status rollout_into(tma_solver *s, const float *d_u, int64_t L, int32_t J, float *cbar,
@@ -1659,7 +1658,7 @@ static bool same_shape(const tma_problem &a, const tma_problem &b)
 // for the whole batch, draws each particle's field in the rollout instead).
 static tma_status batch_wind(tma_batch *b, cudaStream_t st)
 {
-    const size_t P = (size_t)b->probs[0].grid[0] * b->probs[0].grid[1] * b->probs[0].grid[2];
+    const size_t P = (size_t)b->pc_h[0].P;
     for (size_t g = 0; g < b->wind_groups.size() && b->probs[0].wind_mode == 0; ++g) {
         const WindC &w = b->wind_groups[g];
         const int s0 = b->group_start[g];
@@ -1831,7 +1830,8 @@ tma_status tma_batch_create(const tma_problem *probs, const tma_aircraft *const 
         b->J_max = p0.J_max;
         b->sep_mode = p0.sep_mode;
         const int nx = p0.grid[0], ny = p0.grid[1], nz = p0.grid[2], nxy = nx * ny;
-        const size_t P = (size_t)nxy * nz;
+        const WindLayout wl = wind_layout(nx, ny, nz);
+        const size_t P = (size_t)wl.P;
         const long long nLb = ((long long)p0.L + kTileParticles - 1) / kTileParticles;
         auto fail = [&](cudaError_t e) {
             batch_free(b);
@@ -1926,6 +1926,8 @@ tma_status tma_batch_create(const tma_problem *probs, const tma_aircraft *const 
             w.M = nsc * p0.M;
             w.H = p0.H;
             w.nxy = nxy;
+            w.ny = ny;
+            w.out = wl;
             w.nz = nz;
             w.ncol = (int)(nsc * per_scen);
             w.ldb = max_ldb;

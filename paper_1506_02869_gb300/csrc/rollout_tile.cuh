@@ -22,7 +22,10 @@ constexpr float kPi = 3.14159265358979323846f;
 // Trilinear interpolation of one wind field (Sec. 3.9.1) at a position clamped
 // into the grid box: wind_fetch locates the cell and loads its four packed
 // columns (float4 per node: own (x, y) value and the difference to the node one
-// level up), wind_interp combines them.
+// level up; WindLayout), wind_interp combines them.  These four gathers bound the
+// rollout: with a node's levels side by side (8 x 16 bytes), the lanes of a warp,
+// one aircraft at one level, hit one bank group and took about 90 L1 wavefronts
+// per step.
 struct WindFetch {
     float4 a00, a01, a10, a11;
     float tx, ty, tz;
@@ -42,14 +45,13 @@ __device__ __forceinline__ WindFetch wind_fetch(const ProblemC &P, const float4 
         idx[d] = i;
         t[d] = f - (float)i;
     }
-    const int nz = P.grid[2];
-    const int nyz = P.grid[1] * nz;
-    const int p = (idx[0] * P.grid[1] + idx[1]) * nz + idx[2];
+    const float4 *c = Wk + (idx[2] * P.plane + idx[0] * P.pitch + idx[1]);
     WindFetch r;
-    r.a00 = __ldg(Wk + p);
-    r.a01 = __ldg(Wk + p + nz);
-    r.a10 = __ldg(Wk + p + nyz);
-    r.a11 = __ldg(Wk + p + nyz + nz);
+    r.a00 = __ldg(c);
+    r.a01 = __ldg(c + 1);
+    c += P.pitch;
+    r.a10 = __ldg(c);
+    r.a11 = __ldg(c + 1);
     r.tx = t[0];
     r.ty = t[1];
     r.tz = t[2];

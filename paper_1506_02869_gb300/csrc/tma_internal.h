@@ -19,6 +19,28 @@ constexpr int kHalfVariantBase = 13; // first rollout variant index of the 16-pa
 constexpr int kQuarterVariantBase = 16; // first rollout variant index of the 8-particle tile
 constexpr int kMaxRolloutVariants = 24;
 
+// Packed wind field of one (sample, step) as the rollouts read it: a float4 per
+// node (its value and the difference to the node one level up), levels outermost,
+// y innermost, the top level left out (no cell starts there).  Row pitch and
+// level stride are 3 or 5 modulo 8 records (128 bytes are 8 of them): the
+// particles of one aircraft fly at one level in neighbouring cells, and with these
+// strides their 16-byte loads spread over the L1's banks.
+struct WindLayout {
+    int pitch, plane, P;   // records per x row, per level, per field
+};
+inline WindLayout wind_layout(int nx, int ny, int nz)
+{
+    const auto odd = [](int v) {
+        while (v % 8 != 3 && v % 8 != 5) ++v;
+        return v;
+    };
+    WindLayout w;
+    w.pitch = odd(ny);
+    w.plane = odd(nx * w.pitch);
+    w.P = w.plane * (nz - 1);
+    return w;
+}
+
 // Per-aircraft constants in FP32 (derived on the host in FP64).
 struct AircraftC {
     int type;              // 0 arrival, 1 departure
@@ -34,7 +56,8 @@ struct AircraftC {
 struct ProblemC {
     int N, H, S, M, G;     // G = lanes per (particle, sample) group = next_pow2(N)
     int seg_q, seg_r;      // H = seg_q S + seg_r: the control segments' lengths step by these
-    int P;                 // wind grid nodes
+    int P;                 // records of one wind field (WindLayout)
+    int pitch, plane;      // its strides: records per x row, per level
     int grid[3];
     float dt;
     float box_lo[3], box_hi[3], inv_h[3];
@@ -77,6 +100,8 @@ struct DynState {
 // Parameters of the wind-field generation kernels.
 struct WindC {
     int M, H, nxy, nz, ncol, ldb;
+    int ny;
+    WindLayout out;
     uint32_t stream;       // random stream of the normals: 3, or 8 for held-out samples
     float a, b, sigma;
     float Lz[TMA_MAX_GRID_Z * TMA_MAX_GRID_Z];
@@ -113,8 +138,10 @@ struct SegKey {
 
 cudaError_t launch_wind_normals_ar(const WindC &w, const DynState *dyn, float *Btmp,
                                    cudaStream_t st);
-cudaError_t launch_wind_gemm(const WindC &w, const float *Lxy, int lda, const float *Btmp,
-                             float *W, cudaStream_t st);
+// Lxy_t: the horizontal factor transposed, [lda][lda] zero-padded; W_own: the plain
+// values [M][H][nxy][nz][2] too, or nullptr
+cudaError_t launch_wind_gemm(const WindC &w, const float *Lxy_t, int lda, const float *Btmp,
+                             float *W, cudaStream_t st, float *W_own = nullptr);
 
 cudaError_t launch_rollout(const ProblemC &P, const DynState *dyn, const float *u, const float *W,
                            int64_t L, int J, float *cost_ms, float *cost_ms_soft,

@@ -7,145 +7,166 @@
 // over k and applies the small vertical factor L_z, writing
 // Btmp[q][((m H + k) nz + iz) 2 + c] for horizontal node q.
 // Kernel 2 applies the horizontal factor as one lower-triangular matrix
-// product over q (an FP32 register-tiled GEMM) and scatters into the
-// rollout's packed layout: float4 per node; kernel 3 turns the upper half of
-// every record into the difference to the node one level up, so that the
-// trilinear interpolation needs four aligned 16-byte loads and no subtraction
-// in the vertical direction.
-#include "device_common.cuh"
-#include "tma_internal.h"
+// product over q (an FP32 register-tiled GEMM) and writes the rollout's packed
+// layout: float4 per node, its own value and the difference to the node one
+// level up, so that the trilinear interpolation needs four aligned 16-byte
+// loads and no subtraction in the vertical direction; the plain values too
+// when the caller wants them.
+#include "wind_normals.cuh"
 
 namespace tma {
 
 namespace {
 
-__global__ void __launch_bounds__(128) wind_normals_ar_kernel(const WindC w,
-                                                              const DynState *__restrict__ dyn,
+template <int LANES>
+__global__ void __launch_bounds__(128) wind_normals_ar_kernel(const WindC w, const DynState *__restrict__ dyn,
                                                               float *__restrict__ Btmp)
 {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)w.M * w.nxy) return;
-    const int m = (int)(t / w.nxy);
-    const int q = (int)(t - (long long)m * w.nxy);
-    const uint32_t mpc = dyn->mpc_step;
-    const int nz = w.nz;
-    float B[2][TMA_MAX_GRID_Z];
-#pragma unroll
-    for (int iz = 0; iz < TMA_MAX_GRID_Z; ++iz) B[0][iz] = B[1][iz] = 0.0f;
-    float *row = Btmp + (size_t)q * w.ldb;
-    for (int k = 0; k < w.H; ++k) {
-#pragma unroll
-        for (int iz = 0; iz < TMA_MAX_GRID_Z; ++iz) {
-            if (iz < nz) {
-                const uint4 r = draw(w.key0, w.key1, (uint32_t)(q * nz + iz), (uint32_t)m << 8,
-                                     (uint32_t)k, w.stream, 0u, mpc);
-                const float2 n = box_muller(r.x, r.y);
-                if (k == 0) {
-                    B[0][iz] = n.x;
-                    B[1][iz] = n.y;
-                } else {
-                    B[0][iz] = fmaf(w.a, B[0][iz], w.b * n.x);
-                    B[1][iz] = fmaf(w.a, B[1][iz], w.b * n.y);
-                }
-            }
-        }
-        float *o = row + ((size_t)m * w.H + k) * (size_t)(2 * nz);
-#pragma unroll
-        for (int iz = 0; iz < TMA_MAX_GRID_Z; ++iz) {
-            if (iz < nz) {
-                float ax = 0.0f, ay = 0.0f;
-#pragma unroll
-                for (int jz = 0; jz <= iz; ++jz) {
-                    const float lz = w.Lz[iz * TMA_MAX_GRID_Z + jz];
-                    ax = fmaf(lz, B[0][jz], ax);
-                    ay = fmaf(lz, B[1][jz], ay);
-                }
-                o[2 * iz] = ax;
-                o[2 * iz + 1] = ay;
-            }
-        }
-    }
+    const long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+    const int iz = threadIdx.x % LANES;
+    const bool on = t < (long long)w.M * w.nxy && iz < w.nz;
+    const long long tc = min(t, (long long)w.M * w.nxy - 1);
+    const int m = (int)(tc / w.nxy);
+    const int q = (int)(tc - (long long)m * w.nxy);
+    wind_normals_column<LANES>(w, w.key0, w.key1, w.stream, dyn->mpc_step, m, q, iz, on,
+                               Btmp + (size_t)q * w.ldb + (size_t)m * w.H * (size_t)(2 * w.nz));
 }
 
-// C[p][col] = sum_{q <= p} A[p][q] Btmp[q][col]; W[(col / 2nz) nxy + p][col % 2nz] = sigma C.
-// 128 x 128 tiles, K step 8, 8 x 8 outputs per thread.  A is zero-padded to a
-// multiple of 128 rows and lda columns; Btmp is zero-padded to a multiple of 8
-// rows and ldb (multiple of 128) columns, so the main loop needs no guards.
-__global__ void __launch_bounds__(256) wind_gemm_kernel(const WindC w, const float *__restrict__ A,
-                                                        int lda, const float *__restrict__ Bm,
-                                                        float *__restrict__ W)
+__device__ __forceinline__ void cp_async16(float *dst, const float *src, bool on)
 {
-    __shared__ __align__(16) float As[8][128];
-    __shared__ __align__(16) float Bs[8][128];
+    // zero-filled when off
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(on ? 16 : 0)
+                 : "memory");
+}
+
+// Columns of a tile that are used: whole vertical columns of nodes (2 nz values
+// each, so that a node's upper neighbour is in the tile) and a multiple of 4
+// (16-byte copies).
+__host__ __device__ constexpr int wind_tile_cols(int T, int nz)
+{
+    const int unit = nz % 2 == 0 ? 2 * nz : 4 * nz;
+    return T / unit * unit;
+}
+
+// C[p][col] = sum_{q <= p} At[q][p] Btmp[q][col], q ascending in one chain of
+// fused multiply-adds per output, sigma C into the packed layout.  T x T tiles,
+// 8 x 8 outputs per thread (T = 128: 256 threads, T = 64: 64), K in steps of 8
+// through a ring of four stages filled by cp.async; a pair of columns per
+// two-lane FP32 instruction (each lane the IEEE single operation), which halves
+// the issue slots of the products.  At is the factor transposed and zero-padded
+// to multiples of 128, Btmp zero-padded to as many rows, so the main loop needs
+// guards for the last columns only.  Row tiles run from the last (longest sums)
+// to the first.  Bound: the FP32 units (2.6e11 products and sums for 16 samples of
+// a 64 x 64 x 8 grid over 60 steps, 3.2 ms at their peak): that field with its
+// plain values takes 4.57 ms (normals included) against 9.47 ms with a
+// single-buffered loop, a second pass that formed the differences and a strided
+// copy for the plain values.
+constexpr int kStages = 4, kKStep = 8;
+
+template <int T>
+__global__ void __launch_bounds__(T *T / 64, T == 128 ? 2 : 6)
+    wind_gemm_kernel(const WindC w, const float *__restrict__ At, int lda, const float *__restrict__ Bm, int n_ctiles,
+                     int n_rtiles, float4 *__restrict__ W, float2 *__restrict__ Wown)
+{
+    constexpr int kThreads = T * T / 64, kPad = T + 2;   // rows an odd number of 8-byte words apart: no bank conflicts along rows
+    constexpr int kRing = kStages * kKStep * 2 * T, kOut = 64 * kPad;
+    __shared__ __align__(16) float sh[kRing > kOut ? kRing : kOut];
     const int t = threadIdx.x;
-    const int tx = t & 15, ty = t >> 4;
-    const int row0 = blockIdx.y * 128, col0 = blockIdx.x * 128;
-    const int kend = min(((w.nxy + 7) / 8) * 8, row0 + 128);
-    float acc[8][8];
+    const int tx = t % (T / 8), ty = t / (T / 8);
+    const int rt = n_rtiles - 1 - (int)(blockIdx.x / n_ctiles);
+    const int cols = wind_tile_cols(T, w.nz);
+    const int row0 = rt * T, col0 = (int)(blockIdx.x % n_ctiles) * cols;
+    const int steps = (min(w.nxy, row0 + T) + kKStep - 1) / kKStep;
+    float2 acc[8][4];
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
+        for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.0f, 0.0f);
 
-    const int ar = t >> 1, ak = (t & 1) * 4;     // A tile: row ar, k offset ak
-    const int bk = t >> 5, bc = (t & 31) * 4;    // B tile: k row bk, column offset bc
-    for (int k0 = 0; k0 < kend; k0 += 8) {
-        const float4 av = __ldg(reinterpret_cast<const float4 *>(A + (size_t)(row0 + ar) * lda + k0 + ak));
-        const float4 bv = __ldg(reinterpret_cast<const float4 *>(Bm + (size_t)(k0 + bk) * w.ldb + col0 + bc));
-        As[ak + 0][ar] = av.x;
-        As[ak + 1][ar] = av.y;
-        As[ak + 2][ar] = av.z;
-        As[ak + 3][ar] = av.w;
-        *reinterpret_cast<float4 *>(&Bs[bk][bc]) = bv;
-        __syncthreads();
+    // stage s: A rows [kKStep][T], then B rows [kKStep][T]
+    auto fill = [&](int step) {
+        if (step < steps) {
+            float *A = sh + (step % kStages) * kKStep * 2 * T, *B = A + kKStep * T;
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-            const float4 a0 = *reinterpret_cast<const float4 *>(&As[kk][ty * 8]);
-            const float4 a1 = *reinterpret_cast<const float4 *>(&As[kk][ty * 8 + 4]);
-            const float4 b0 = *reinterpret_cast<const float4 *>(&Bs[kk][tx * 4]);
-            const float4 b1 = *reinterpret_cast<const float4 *>(&Bs[kk][64 + tx * 4]);
-            const float ar8[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float br8[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+            for (int e = t; e < kKStep * T / 4; e += kThreads) {
+                const int k = e / (T / 4), c = e % (T / 4) * 4;
+                const size_t q = (size_t)(step * kKStep + k);
+                cp_async16(A + k * T + c, At + q * lda + row0 + c, true);
+                const bool on = col0 + c < w.ldb;
+                cp_async16(B + k * T + c, Bm + q * w.ldb + (on ? col0 + c : 0), on);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int s = 0; s < kStages - 1; ++s) fill(s);
+    for (int step = 0; step < steps; ++step) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+        __syncthreads();                 // this step's stage is filled, the previous step's is free
+        fill(step + kStages - 1);
+        const float *A = sh + (step % kStages) * kKStep * 2 * T + ty * 8;
+        const float *B = sh + (step % kStages) * kKStep * 2 * T + kKStep * T + tx * 4;
+#pragma unroll
+        for (int kk = 0; kk < kKStep; ++kk) {
+            const float4 a0 = *reinterpret_cast<const float4 *>(A + kk * T);
+            const float4 a1 = *reinterpret_cast<const float4 *>(A + kk * T + 4);
+            const float4 b0 = *reinterpret_cast<const float4 *>(B + kk * T);
+            const float4 b1 = *reinterpret_cast<const float4 *>(B + kk * T + T / 2);
+            const float ar[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float2 br[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                                  make_float2(b1.z, b1.w)};
 #pragma unroll
             for (int a = 0; a < 8; ++a)
 #pragma unroll
-                for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(ar8[a], br8[b], acc[a][b]);
+                for (int b = 0; b < 4; ++b) acc[a][b] = __ffma2_rn(make_float2(ar[a], ar[a]), br[b], acc[a][b]);
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+
+    // through shared memory, 64 rows at a time, into the packed records: for each
+    // field mk and level, consecutive threads take consecutive rows (nodes along y)
+    const int two_nz = 2 * w.nz;
+    const int mk0 = col0 / two_nz, n_mk = min(cols, w.ncol - col0) / two_nz;
+    const float sg = w.sigma;
+    for (int h = 0; h < T / 64; ++h) {
+        __syncthreads();
+        if (ty / 8 == h) {
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                float2 *o = reinterpret_cast<float2 *>(sh + (ty % 8 * 8 + a) * kPad + tx * 4);
+                o[0] = acc[a][0];
+                o[1] = acc[a][1];
+                o[T / 4] = acc[a][2];
+                o[T / 4 + 1] = acc[a][3];
+            }
         }
         __syncthreads();
-    }
-    // scatter into the packed layout: node q of field (m, k) holds
-    // (W_x(q), W_y(q), W_x(q + 1 level), W_y(q + 1 level)); the top level
-    // repeats its own value in the upper half (never read by interpolation)
-    const int two_nz = 2 * w.nz;
-    const int P = w.nxy * w.nz;
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-        const int row = row0 + ty * 8 + a;
-        if (row >= w.nxy) continue;
-#pragma unroll
-        for (int b = 0; b < 8; b += 2) {
-            const int col = col0 + (b < 4 ? tx * 4 + b : 64 + tx * 4 + (b - 4));
-            if (col >= w.ncol) continue;   // ncol is even: a pair (x, y) is never split
-            const int mk = col / two_nz;
-            const int iz = (col - mk * two_nz) >> 1;
-            const float2 val = make_float2(w.sigma * acc[a][b], w.sigma * acc[a][b + 1]);
-            float2 *rec = reinterpret_cast<float2 *>(W + ((size_t)mk * P + (size_t)row * w.nz + iz) * 4);
-            rec[0] = val;
-            if (iz == w.nz - 1) rec[1] = val;
-            if (iz > 0) rec[-1] = val;      // upper half of the record one level below
+        const int r0 = row0 + h * 64, rows = min(64, w.nxy - r0);
+        const int row = t % 64, p = r0 + row;
+        if (row < rows) {
+            const size_t rec = (size_t)(p / w.ny) * w.out.pitch + p % w.ny;
+            const float *src = sh + row * kPad;
+            for (int c = t / 64; c < n_mk * (w.nz - 1); c += kThreads / 64) {
+                const int mk = c / (w.nz - 1), iz = c - mk * (w.nz - 1);
+                const float2 lo = *reinterpret_cast<const float2 *>(src + mk * two_nz + 2 * iz);
+                const float2 hi = *reinterpret_cast<const float2 *>(src + mk * two_nz + 2 * iz + 2);
+                const float2 own = make_float2(__fmul_rn(sg, lo.x), __fmul_rn(sg, lo.y));
+                W[(size_t)(mk0 + mk) * w.out.P + (size_t)iz * w.out.plane + rec] =
+                    make_float4(own.x, own.y, __fsub_rn(__fmul_rn(sg, hi.x), own.x),
+                                __fsub_rn(__fmul_rn(sg, hi.y), own.y));
+            }
+        }
+        if (Wown) {
+            // the caller's layout [mk][row][level][2]: consecutive threads take consecutive levels
+            for (int n = t; n < n_mk * rows * w.nz; n += kThreads) {
+                const int iz = n % w.nz, q = n / w.nz, mk = q / rows, r = q - mk * rows;
+                const float2 v = *reinterpret_cast<const float2 *>(sh + r * kPad + mk * two_nz + 2 * iz);
+                Wown[((size_t)(mk0 + mk) * w.nxy + r0 + r) * w.nz + iz] =
+                    make_float2(__fmul_rn(sg, v.x), __fmul_rn(sg, v.y));
+            }
         }
     }
-}
-
-// rec = (W_x, W_y, W_x one level up, W_y one level up) -> (W_x, W_y, dW_x, dW_y)
-__global__ void __launch_bounds__(256) wind_diff_kernel(float4 *__restrict__ W, long long n)
-{
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    float4 r = W[t];
-    r.z -= r.x;
-    r.w -= r.y;
-    W[t] = r;
 }
 
 }  // namespace
@@ -153,23 +174,38 @@ __global__ void __launch_bounds__(256) wind_diff_kernel(float4 *__restrict__ W, 
 cudaError_t launch_wind_normals_ar(const WindC &w, const DynState *dyn, float *Btmp,
                                    cudaStream_t st)
 {
-    const long long n = (long long)w.M * w.nxy;
-    if (n <= 0) return cudaSuccess;
-    wind_normals_ar_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(w, dyn, Btmp);
+    if (w.M <= 0 || w.nxy <= 0) return cudaSuccess;
+    const int lanes = wind_column_lanes(w.nz);
+    const unsigned grid = (unsigned)(((long long)w.M * w.nxy * lanes + 127) / 128);
+    switch (lanes) {
+    case 2: wind_normals_ar_kernel<2><<<grid, 128, 0, st>>>(w, dyn, Btmp); break;
+    case 4: wind_normals_ar_kernel<4><<<grid, 128, 0, st>>>(w, dyn, Btmp); break;
+    case 8: wind_normals_ar_kernel<8><<<grid, 128, 0, st>>>(w, dyn, Btmp); break;
+    default: wind_normals_ar_kernel<16><<<grid, 128, 0, st>>>(w, dyn, Btmp); break;
+    }
     count_launch();
     return cudaGetLastError();
 }
 
-cudaError_t launch_wind_gemm(const WindC &w, const float *Lxy, int lda, const float *Btmp,
-                             float *W, cudaStream_t st)
+cudaError_t launch_wind_gemm(const WindC &w, const float *Lxy_t, int lda, const float *Btmp,
+                             float *W, cudaStream_t st, float *W_own)
 {
-    dim3 grid(w.ldb / 128, (w.nxy + 127) / 128);
-    wind_gemm_kernel<<<grid, 256, 0, st>>>(w, Lxy, lda, Btmp, W);
-    count_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const long long n = (long long)(w.ncol / (2 * w.nz)) * w.nxy * w.nz;   // records
-    wind_diff_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(reinterpret_cast<float4 *>(W), n);
+    const auto tiles = [&](int T, int &ct, int &rt) {
+        const int cols = wind_tile_cols(T, w.nz);
+        ct = (w.ncol + cols - 1) / cols;
+        rt = (w.nxy + T - 1) / T;
+    };
+    int ct, rt;
+    tiles(128, ct, rt);
+    float4 *W4 = reinterpret_cast<float4 *>(W);
+    float2 *W2 = reinterpret_cast<float2 *>(W_own);
+    // fewer 128 x 128 tiles than two per SM: 64 x 64 tiles keep the chip busier
+    if ((long long)ct * rt >= 2 * 152) {
+        wind_gemm_kernel<128><<<ct * rt, 256, 0, st>>>(w, Lxy_t, lda, Btmp, ct, rt, W4, W2);
+    } else {
+        tiles(64, ct, rt);
+        wind_gemm_kernel<64><<<ct * rt, 64, 0, st>>>(w, Lxy_t, lda, Btmp, ct, rt, W4, W2);
+    }
     count_launch();
     return cudaGetLastError();
 }
