@@ -115,14 +115,14 @@ ROLLOUT_TRAFFIC = {"sources_sha256_16": "9c6681ad7c36f584",
 
 
 def rollout_kernel_name(variant):
-    """The rollout kernel a launch variant runs (8-12: two wind samples per thread; 13-15 and
+    """The rollout kernel a launch variant runs (8-12 and 18-19: the two-kernel form; 13-15 and
     16-17 the one-sample kernel on 16- and 8-particle tiles)."""
-    return "rollout_pair_kernel" if variant is not None and 8 <= variant < 13 else "rollout_kernel"
+    return "wind_rollout_kernel" if variant is not None and (8 <= variant < 13 or variant >= 18) else "rollout_kernel"
 
 
 def rollout_sources_digest():
     h = hashlib.sha256()
-    for f in ("rollout.cu", "rollout_pair.cu", "rollout_tile.cuh", "device_common.cuh"):
+    for f in ("rollout.cu", "rollout_traj.cu", "rollout_tile.cuh", "device_common.cuh"):
         with open(os.path.join(ROOT, "paper_1506_02869_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -996,15 +996,13 @@ def run_layout_sweep(args, local):
     draws = sum(min(math.floor(3 + 5 * math.exp(0.05 * J)), p.M) for J in range(p.J_max))
     units_settled = p.L * draws * p.N * p.H        # every aircraft active over the whole horizon
     names = {0: "256x4", 1: "256x3", 2: "512x2", 3: "512x1", 4: "1024x1", 5: "256x2",
-             6: "384x2", 7: "768x1", 8: "pair 256x3", 9: "pair 256x2", 10: "pair 384x2",
-             11: "pair 512x1", 12: "pair 768x1"}
-    regs = {0: 64, 1: 85, 2: 64, 3: 128, 4: 64, 5: 128, 6: 85, 7: 85, 8: 85, 9: 128, 10: 85,
-            11: 128, 12: 85}
+             6: "384x2", 7: "768x1", 18: "two kernels 256x4", 19: "two kernels 256x5"}
+    regs = {0: 64, 1: 85, 2: 64, 3: 128, 4: 64, 5: 128, 6: 85, 7: 85, 18: 64, 19: 48}
     stream = torch.cuda.current_stream()
     n_steps = args.mpc_steps if args.mpc_steps > 6 else 9
     rows = []
     auto = None
-    for v in (range(13) if args.variant < 0 else [args.variant]):
+    for v in (list(names) if args.variant < 0 else [args.variant]):
         sol = pkg.Solver(p)
         if auto is None:
             auto = pkg.tma_get_tuning(sol.h)[0]

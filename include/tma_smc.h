@@ -239,8 +239,8 @@ tma_status tma_best_index(tma_solver *s, int64_t *h_best, tma_stream_t stream);
 
 /* Launch configuration of the rollout kernel chosen by the autotuner that
  * tma_create runs (Sec. 4.4 sweeps thread/block layouts by hand; here every
- * valid launch-bound variant -- block-size cap and minimum resident blocks --
- * is timed on the solver's own workload and the fastest kept; the choice is
+ * the launch-bound variants -- block-size cap and minimum resident blocks -- that
+ * can be the fastest are timed on the solver's own workload and the fastest kept; the choice is
  * cached per device, aircraft count, problem kind and workload size class).
  * *n_timed is 0 when the choice came from the cache; h_variants/h_ms (up to 24
  * entries, may be NULL) receive the
@@ -251,11 +251,13 @@ tma_status tma_get_tuning(tma_solver *s, int32_t *variant, int32_t *n_timed, int
 /* Force the rollout kernel's launch variant for this solver, e.g. to sweep
  * the layouts as Sec. 4.4 does.  0-7: one wind sample per thread, block-size
  * cap x minimum resident blocks = 256x4, 256x3, 512x2, 512x1, 1024x1, 256x2,
- * 384x2, 768x1.  8-12: two wind samples per thread (m and m + ceil(M/2); the
- * wind-independent part of each step -- limits, drag, thrust, fuel, altitude,
- * airspeed, heading -- computed once for both), 256x3, 256x2, 384x2, 512x1,
- * 768x1; only for the shared wind field (wind mode 0) without the rolling
- * window and M >= 2.  13-15: the one-sample kernel on tiles of 16 particles (a
+ * 384x2, 768x1.  18-19: the two-kernel rollout (what does not depend on the wind
+ * -- limits, drag, thrust, fuel, altitude, airspeed, heading, vertical
+ * separation -- computed once per particle, the rest per sample), 256x4 and
+ * 256x5, for M >= 2 and where memory for its workspace (at most 512 MB) was at
+ * hand at creation.  8-12: older names of 18, for the shared wind field (wind
+ * mode 0) without the rolling window and block caps 256, 256, 384, 512, 768 at
+ * 32 N threads.  13-15: the one-sample kernel on tiles of 16 particles (a
  * warp holds two aircraft; block 16 N threads), 768x1, 384x2, 512x2; 16-17: on
  * tiles of 8 particles (four aircraft per warp; block 8 N threads), 512x2,
  * 384x2; both for the shared wind field only and for N a multiple of 2 or 4

@@ -233,6 +233,7 @@ static ProblemC derive_problem(const tma_problem &p, const tma_aircraft *aircraf
         P.box_lo[d] = (float)p.box_lo[d];
         P.box_hi[d] = (float)p.box_hi[d];
         P.inv_h[d] = (float)((p.grid[d] - 1) / (p.box_hi[d] - p.box_lo[d]));
+        P.cell_cap[d] = 8388608.0f + (float)(p.grid[d] - 2);
     }
     P.dt = (float)p.dt;
     P.wind_mode = p.wind_mode;
@@ -359,7 +360,7 @@ static void free_all(tma_solver *s)
                     s->d_live, s->d_best_u, s->d_probs1, s->d_scen1, s->d_seg_scen1,
                     s->d_gcost_ms, s->d_gpart, s->d_eps, s->d_nacc, s->d_acc_hist,
                     s->d_eps_hist, s->d_u_prop, s->d_grad0, s->d_grad1, s->d_cbar0, s->d_cbar1,
-                    s->d_cost0, s->d_cost1, s->d_inbox};
+                    s->d_cost0, s->d_cost1, s->d_inbox, s->d_traj};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -368,6 +369,24 @@ template <typename T>
 static cudaError_t alloc(T **p, size_t bytes)
 {
     return cudaMalloc(reinterpret_cast<void **>(p), bytes > 0 ? bytes : 16);
+}
+
+// A buffer that only saves time: beyond 64 MB it is taken only when it is at most
+// a sixteenth of the free memory, so that what needed the memory without it still
+// gets it.
+static bool alloc_spare(void **p, size_t bytes)
+{
+    *p = nullptr;
+    if (bytes == 0) return false;
+    size_t free_b = 0, total_b = 0;
+    const bool fits = bytes <= ((size_t)64 << 20) ||
+                      (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 16);
+    if (!fits || cudaMalloc(p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        *p = nullptr;
+        return false;
+    }
+    return true;
 }
 
 // Static (FP32) copies of the control box and move sigma.
@@ -477,25 +496,26 @@ static std::string tune_key_of(const tma_problem &p, int device)
 static std::string tune_key(const tma_solver *s) { return tune_key_of(s->prob, s->device); }
 
 // Times every launch variant of the rollout kernel valid for P on the given
-// buffers (Lp particles, all wind samples, iteration 0, the hard costs only):
-// one untimed launch and three timed per variant; *best = the fastest, and the
+// buffers (Lp particles, all wind samples, iteration 0, the soft costs too when
+// the problem has them): one untimed launch and three timed per variant; *best = the fastest, and the
 // timings in tv[] / tms[] (*nt entries).
 static cudaError_t time_rollout_variants(const ProblemC &P, const DynState *dyn, const float *u,
-                                         const float *W, int64_t Lp, float *cost, cudaStream_t st,
-                                         cudaEvent_t e0, cudaEvent_t e1, int *best, int *nt, int *tv,
+                                         const float *W, int64_t Lp, float *cost, float *cost_soft, void *ws, size_t ws_bytes,
+                                         cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int *best, int *nt, int *tv,
                                          float *tms)
 {
     int cand[kMaxRolloutVariants];
-    const int nc = rollout_variants(P, cand);
+    int nc = 0;
+    rollout_variants(P, ws_bytes, cand, &nc);
     *best = cand[0];
     *nt = 0;
     float best_ms = 1e30f;
     cudaError_t e = cudaSuccess;
     for (int c = 0; c < nc && e == cudaSuccess; ++c) {
-        e = launch_rollout(P, dyn, u, W, Lp, 0, cost, nullptr, nullptr, st, cand[c]);
+        e = launch_rollout(P, dyn, u, W, Lp, 0, cost, cost_soft, nullptr, st, cand[c], ws, ws_bytes);
         if (e == cudaSuccess) e = cudaEventRecord(e0, st);
         for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep)
-            e = launch_rollout(P, dyn, u, W, Lp, 0, cost, nullptr, nullptr, st, cand[c]);
+            e = launch_rollout(P, dyn, u, W, Lp, 0, cost, cost_soft, nullptr, st, cand[c], ws, ws_bytes);
         if (e == cudaSuccess) e = cudaEventRecord(e1, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.0f;
@@ -648,6 +668,9 @@ tma_status tma_create(const tma_problem *prob, const tma_aircraft *aircraft, tma
         if ((e = alloc(&s->d_live, 8))) return fail(e);
         if ((e = alloc(&s->d_best_u, N * p.S * 3 * 4))) return fail(e);
         if ((e = alloc(&s->d_dyn, sizeof(DynState)))) return fail(e);
+        // the trajectories' workspace; without it the one-sample kernels run
+        s->traj_bytes = traj_workspace(s->P, p.L);
+        if (!alloc_spare(&s->d_traj, s->traj_bytes)) s->traj_bytes = 0;
         DynState d;
         upload_x0(s, d);
         if ((e = cudaMemcpy(s->d_dyn, &d, sizeof d, cudaMemcpyHostToDevice))) return fail(e);
@@ -706,7 +729,7 @@ tma_status tma_set_tuning(tma_solver *s, int32_t variant)
 {
     if (!s) return TMA_ERR_INVALID_ARG;
     int cand[kMaxRolloutVariants];
-    const int n = rollout_variants(s->P, cand);
+    const int n = rollout_variants(s->P, s->traj_bytes, cand);
     for (int c = 0; c < n; ++c)
         if (cand[c] == variant) {
             s->rollout_variant = variant;
@@ -793,7 +816,7 @@ static tma_status gen_wind(tma_solver *s, cudaStream_t st, float *d_W = nullptr)
 static tma_status autotune_rollout(tma_solver *s)
 {
     int cand[kMaxRolloutVariants];
-    const int nc = rollout_variants(s->P, cand);
+    const int nc = rollout_variants(s->P, s->traj_bytes, cand);
     s->rollout_variant = cand[0];
     s->n_tuned = 0;
     if (nc <= 1) return TMA_OK;
@@ -830,8 +853,8 @@ static tma_status autotune_rollout(tma_solver *s)
     if (r == TMA_OK) {
         e = launch_init_controls(s->P, s->d_dyn, lo, hi, s->d_u[0], Lp, st);
         if (e == cudaSuccess)
-            e = time_rollout_variants(s->P, s->d_dyn, s->d_u[0], s->d_W, Lp, s->d_cost_ms, st, e0, e1,
-                                      &s->rollout_variant, &s->n_tuned, s->tuned_variant, s->tuned_ms);
+            e = time_rollout_variants(s->P, s->d_dyn, s->d_u[0], s->d_W, Lp, s->d_cost_ms, s->d_cost_ms_soft,
+                                      s->d_traj, s->traj_bytes, st, e0, e1, &s->rollout_variant, &s->n_tuned, s->tuned_variant, s->tuned_ms);
         if (e != cudaSuccess) r = cuda_fail(e);
     }
     cleanup();
@@ -873,7 +896,7 @@ static tma_status rollout_into(tma_solver *s, const float *d_u, int64_t L, int32
         StageTimer t(s, 2, st);
         TMA_CUDA(launch_rollout(Pj, s->d_dyn, d_u, s->d_W, L, J, s->d_cost_ms,
                                 soft ? s->d_cost_ms_soft : nullptr, s->d_live, st,
-                                s->rollout_variant));
+                                s->rollout_variant, s->d_traj, s->traj_bytes));
     }
     {
         StageTimer t(s, 3, st);
@@ -1636,7 +1659,7 @@ static void batch_free(tma_batch *b)
                     b->d_Btmp, b->d_W, b->d_u[0], b->d_u[1], b->d_cost_ms, b->d_cost_ms_soft,
                     b->d_cbar, b->d_cbar_soft, b->d_wtilde, b->d_anc, b->d_work, b->d_best,
                     b->d_best_sum, b->d_ninf, b->d_best_u, b->d_t_start, b->d_t_end, b->d_live,
-                    b->d_queue, b->d_flags, b->d_err};
+                    b->d_queue, b->d_flags, b->d_err, b->d_traj};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (float *p : b->d_pops)
@@ -1688,7 +1711,9 @@ static cudaError_t batch_rollout(tma_batch *b, const float *d_u, int J, int Mj, 
         Ps.M = Mj;
         const size_t co = (size_t)sc.seg_off * b->M * (size_t)b->L;
         e = launch_rollout(Ps, b->d_dyns + s, d_u + sc.u_off, b->d_W + (size_t)sc.w_off * 4, b->L, J, cost + co,
-                           cost_soft ? cost_soft + co : nullptr, b->d_live, b->aux[s % ns], b->scen_variant[s]);
+                           cost_soft ? cost_soft + co : nullptr, b->d_live, b->aux[s % ns], b->scen_variant[s],
+                           b->d_traj ? static_cast<char *>(b->d_traj) + (size_t)(s % ns) * b->traj_bytes : nullptr,
+                           b->traj_bytes);
     }
     for (int q = 0; q < ns && e == cudaSuccess; ++q) e = cudaEventRecord(b->join_ev[q], b->aux[q]);
     for (int q = 0; q < ns && e == cudaSuccess; ++q) e = cudaStreamWaitEvent(st, b->join_ev[q], 0);
@@ -1772,7 +1797,9 @@ static tma_status batch_tune(tma_batch *b)
         int best = 0, nt = 0, tv[kMaxRolloutVariants];
         float tms[kMaxRolloutVariants];
         e = time_rollout_variants(b->pc_h[s], b->d_dyns + s, b->d_u[0] + sc.u_off, b->d_W + (size_t)sc.w_off * 4,
-                                  Lp, b->d_cost_ms + (size_t)sc.seg_off * b->M * (size_t)b->L, st, e0, e1, &best,
+                                  Lp, b->d_cost_ms + (size_t)sc.seg_off * b->M * (size_t)b->L,
+                                  b->d_cost_ms_soft ? b->d_cost_ms_soft + (size_t)sc.seg_off * b->M * (size_t)b->L : nullptr,
+                                  b->d_traj, b->traj_bytes, st, e0, e1, &best,
                                   &nt, tv, tms);
         if (e == cudaSuccess) {
             b->scen_variant[s] = best;
@@ -1782,9 +1809,9 @@ static tma_status batch_tune(tma_batch *b)
     }
     const int M0 = samples_of(b->probs[0], 0);
     for (int form = 0; form < 2 && r == TMA_OK && e == cudaSuccess; ++form) {
-        e = batch_rollout(b, b->d_u[0], 0, M0, b->d_cost_ms, nullptr, form, st);
+        e = batch_rollout(b, b->d_u[0], 0, M0, b->d_cost_ms, b->d_cost_ms_soft, form, st);
         if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-        if (e == cudaSuccess) e = batch_rollout(b, b->d_u[0], 0, M0, b->d_cost_ms, nullptr, form, st);
+        if (e == cudaSuccess) e = batch_rollout(b, b->d_u[0], 0, M0, b->d_cost_ms, b->d_cost_ms_soft, form, st);
         if (e == cudaSuccess) e = cudaEventRecord(e1, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         if (e == cudaSuccess) e = cudaEventElapsedTime(&b->dispatch_ms[form], e0, e1);
@@ -1983,6 +2010,11 @@ tma_status tma_batch_create(const tma_problem *probs, const tma_aircraft *const 
             if ((e = cudaEventCreateWithFlags(&b->join_ev[q], cudaEventDisableTiming))) return fail(e);
         }
         if ((e = cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming))) return fail(e);
+        // trajectories of the largest scenario, one workspace per auxiliary
+        // stream (a stream's launches run one after the other)
+        for (const ProblemC &q : pc) b->traj_bytes = std::max(b->traj_bytes, traj_workspace(q, p0.L));
+        b->traj_bytes = (b->traj_bytes + 255) / 256 * 256;
+        if (!alloc_spare(&b->d_traj, b->traj_bytes * tma_batch::kAuxStreams)) b->traj_bytes = 0;
         b->grid = batch_rollout_grid();
         b->pc_h = pc;
     } catch (const std::bad_alloc &) {

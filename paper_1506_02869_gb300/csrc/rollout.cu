@@ -85,18 +85,40 @@ static bool small_tile_valid(const ProblemC &P, int tp, int cap)
     return P.wind_mode == 0 && !P.rolling && P.N % (32 / tp) == 0 && cap >= P.N * tp;
 }
 
-int rollout_variants(const ProblemC &P, int *out)
+// Variants 8-12, the names of an earlier kernel that computed the wind-independent
+// part once for two samples: they run the two-kernel form, for the problems and
+// block caps they always took (shared wind field, no rolling window).
+constexpr int kPairCaps[] = {256, 256, 384, 512, 768};
+constexpr int kNumPairVariants = sizeof(kPairCaps) / sizeof(kPairCaps[0]);
+static_assert(kPairVariantBase + kNumPairVariants <= kHalfVariantBase, "variant table");
+
+int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed)
 {
-    int n = 0;
+    int n = 0, tv[kMaxRolloutVariants];
+    const int nt = rollout_traj_variants(P, ws_bytes, tv);
+    const auto fits = [&](int v) { return kVariants[v].max_threads >= P.N * kPB; };
+    const auto listed = [&](int v) {
+        for (int c = 0; c < n; ++c)
+            if (out[c] == v) return true;
+        return false;
+    };
+    // With the two-kernel form at hand the one-sample kernel is the faster one
+    // only for small work (2 aircraft, 1024 particles, 8 samples: 23 against 33 us),
+    // where its register budget decides: one variant of each is timed.
+    for (int c = 0; c < nt; ++c) out[n++] = kTrajVariantBase + tv[c];
+    for (int v : {3, 7, 4})                      // 128, 85 and 64 registers
+        if (nt > 0 && fits(v)) out[n++] = v;
+    if (n_timed && nt > 0) *n_timed = n;
     for (int v = 0; v < kNumVariants; ++v)
-        if (kVariants[v].max_threads >= P.N * kPB) out[n++] = v;
-    int pv[kMaxRolloutVariants];
-    const int np = rollout_pair_variants(P, pv);
-    for (int c = 0; c < np; ++c) out[n++] = kPairVariantBase + pv[c];
+        if (fits(v) && !listed(v)) out[n++] = v;
     for (int v = 0; v < kNumHalfVariants; ++v)
         if (small_tile_valid(P, 16, kHalfVariants[v].max_threads)) out[n++] = kHalfVariantBase + v;
     for (int v = 0; v < kNumQuarterVariants; ++v)
         if (small_tile_valid(P, 8, kQuarterVariants[v].max_threads)) out[n++] = kQuarterVariantBase + v;
+    if (n_timed && nt == 0) *n_timed = n;
+    if (nt > 0 && P.wind_mode == 0 && !P.rolling)
+        for (int v = 0; v < kNumPairVariants; ++v)
+            if (kPairCaps[v] >= P.N * kPB) out[n++] = kPairVariantBase + v;
     return n;
 }
 
@@ -127,9 +149,17 @@ static void launch_small_tile(const ProblemC &P, const DynState *dyn, const floa
 
 cudaError_t launch_rollout(const ProblemC &P, const DynState *dyn, const float *u, const float *W,
                            int64_t L, int J, float *cost_ms, float *cost_ms_soft,
-                           unsigned long long *live, cudaStream_t st, int variant)
+                           unsigned long long *live, cudaStream_t st, int variant, void *ws, size_t ws_bytes)
 {
     if (L <= 0) return cudaSuccess;
+    if (variant >= kTrajVariantBase || (variant >= kPairVariantBase && variant < kHalfVariantBase)) {
+        int tv[kMaxRolloutVariants];
+        const int nt = rollout_traj_variants(P, ws_bytes, tv);
+        const int v = variant >= kTrajVariantBase ? variant - kTrajVariantBase : 0;
+        if (v < nt)
+            return launch_rollout_traj(P, dyn, u, W, L, J, cost_ms, cost_ms_soft, live, st, v, ws, ws_bytes);
+        variant = -1;                  // not valid for this problem: the one-sample kernel
+    }
     if (variant >= kHalfVariantBase) {
         const float4 *W4 = reinterpret_cast<const float4 *>(W);
         const int hv = variant - kHalfVariantBase, qv = variant - kQuarterVariantBase;
@@ -150,17 +180,10 @@ cudaError_t launch_rollout(const ProblemC &P, const DynState *dyn, const float *
             return cudaGetLastError();
         }
         variant = -1;                  // not valid for this problem: the one-sample kernel
-    } else if (variant >= kPairVariantBase) {
-        int pv[kMaxRolloutVariants];
-        const int np = rollout_pair_variants(P, pv);
-        for (int c = 0; c < np; ++c)
-            if (pv[c] == variant - kPairVariantBase)
-                return launch_rollout_pair(P, dyn, u, W, L, J, cost_ms, cost_ms_soft, live, st, pv[c]);
-        variant = -1;                  // not valid for this problem: the one-sample kernel
     }
     if (variant < 0 || variant >= kNumVariants || kVariants[variant].max_threads < P.N * kPB) {
         int cand[kMaxRolloutVariants];
-        rollout_variants(P, cand);
+        rollout_variants(P, 0, cand);
         variant = cand[0];
     }
     const long long nLb = (L + kPB - 1) / kPB;

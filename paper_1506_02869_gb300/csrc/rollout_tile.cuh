@@ -31,30 +31,38 @@ struct WindFetch {
     float tx, ty, tz;
 };
 
-__device__ __forceinline__ WindFetch wind_fetch(const ProblemC &P, const float4 *__restrict__ Wk,
-                                                float x, float y, float z)
+// Cell index and fraction of one coordinate on its grid axis.  The floor of the
+// grid coordinate f in [0, n - 1] comes from one addition of 2^23 rounded toward
+// zero: its low mantissa bits are the integer, subtracting 2^23 again gives it
+// as FP32, so neither conversion goes through the quarter-rate unit (the same
+// integer as (int)f; the cap n - 2 is applied to the sum, where it is exact).
+__device__ __forceinline__ int grid_cell(const ProblemC &P, int d, float pos, float &t)
 {
-    const float pos[3] = {x, y, z};
-    int idx[3];
-    float t[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const float c = fminf(fmaxf(pos[d], P.box_lo[d]), P.box_hi[d]);
-        const float f = (c - P.box_lo[d]) * P.inv_h[d];
-        const int i = min((int)f, P.grid[d] - 2);
-        idx[d] = i;
-        t[d] = f - (float)i;
-    }
-    const float4 *c = Wk + (idx[2] * P.plane + idx[0] * P.pitch + idx[1]);
-    WindFetch r;
+    const float c = fminf(fmaxf(pos, P.box_lo[d]), P.box_hi[d]);
+    const float f = (c - P.box_lo[d]) * P.inv_h[d];
+    const float y = fminf(__fadd_rz(f, 8388608.0f), P.cell_cap[d]);
+    t = f - (y - 8388608.0f);
+    return __float_as_int(y) - 0x4B000000;
+}
+
+// The cell's columns (lower corner in all three axes at ix, iy, iz).
+__device__ __forceinline__ void wind_columns(const ProblemC &P, const float4 *__restrict__ Wk, int ix, int iy,
+                                             int iz, WindFetch &r)
+{
+    const float4 *c = Wk + (iz * P.plane + ix * P.pitch + iy);
     r.a00 = __ldg(c);
     r.a01 = __ldg(c + 1);
     c += P.pitch;
     r.a10 = __ldg(c);
     r.a11 = __ldg(c + 1);
-    r.tx = t[0];
-    r.ty = t[1];
-    r.tz = t[2];
+}
+
+__device__ __forceinline__ WindFetch wind_fetch(const ProblemC &P, const float4 *__restrict__ Wk,
+                                                float x, float y, float z)
+{
+    WindFetch r;
+    const int ix = grid_cell(P, 0, x, r.tx), iy = grid_cell(P, 1, y, r.ty), iz = grid_cell(P, 2, z, r.tz);
+    wind_columns(P, Wk, ix, iy, iz, r);
     return r;
 }
 
@@ -276,6 +284,71 @@ struct CostSums {
     }
 };
 
+// Control segment of step k: segment s covers the steps [ceil(s H / S),
+// ceil((s + 1) H / S)) (every segment has a step: S <= H); knext = ceil((seg + 1)
+// H / S) advances by H = seg_q S + seg_r with its remainder carried, so no
+// division (a late entrant passes several segments at its first step).
+__device__ __forceinline__ void segment_advance(const ProblemC &P, AcState &s, const float *__restrict__ ul, int k)
+{
+    if (k < s.knext) return;
+    do {
+        ++s.seg;
+        s.knext += P.seg_q;
+        s.srem += P.seg_r;
+        if (s.srem >= P.S) {
+            s.srem -= P.S;
+            ++s.knext;
+        }
+    } while (k >= s.knext);
+    s.ks = k;
+    s.uw = __ldg(ul + 3 * s.seg);
+    s.uh = __ldg(ul + 3 * s.seg + 1);
+    s.ua = __ldg(ul + 3 * s.seg + 2);
+    s.zb = s.z;
+    s.vb = s.v;
+    s.cb = s.chi;
+}
+
+// Control-derived quantities of the step-k state and their limits (Sec. 3.4):
+// cos(gamma) and the thrust; false when a limit fails.
+__device__ __forceinline__ bool control_limits(const ProblemC &P, const AircraftC &A, const AcState &s,
+                                               float m0, float &cg, float &T)
+{
+    const float mass = m0 - s.F.s;
+    const float sg = __fdividef(s.uh, s.v);
+    bool ok = fabsf(sg) <= P.sgmax;
+    cg = sqrtf(fmaxf(1.0f - sg * sg, 0.0f));
+    const float tp = __fdividef(s.uw * s.v, kG0 * cg);
+    ok = ok && (fabsf(tp) < P.tpmax);
+    const float secphi = sqrtf(fmaf(tp, tp, 1.0f));
+    const float rho = 1.225f * ex2_approx(4.2559f * __log2f(fmaxf(fmaf(-2.2558e-5f, s.z, 1.0f), 1e-30f)));
+    const float qS = A.halfS * rho * s.v * s.v;
+    const float CL = __fdividef(mass * kG0 * cg * secphi, qS);
+    const float D = qS * fmaf(A.CD2, CL * CL, A.CD0);
+    T = fmaf(mass, fmaf(kG0, sg, s.ua), D);
+    return ok && (T >= A.Tmin) && (T <= A.Tmax);
+}
+
+// The wind-independent part of the Euler step of Eq. (hor); v sin(gamma) =
+// hdot, the speed equation reduces to v += dt a and the heading equation to
+// chi += dt w (coordinated turn).  Within a control segment z, v and chi are
+// linear in time: they are evaluated from the segment's start values so that
+// rounding does not accumulate.  Returns whether the new state is within the
+// unary limits.
+__device__ __forceinline__ bool air_advance(const ProblemC &P, const AircraftC &A, AcState &s, float m0, int k,
+                                            float T)
+{
+    const float dt = P.dt;
+    const float nk = (float)(k + 1 - s.ks) * dt;
+    s.z = fmaf(nk, s.uh, s.zb);
+    const float eta = A.Cf1 * fmaf(s.v, A.invCf2, 1.0f);
+    s.F.add(dt * eta * T);
+    s.v = fmaf(nk, s.ua, s.vb);
+    s.chi = fmaf(nk, s.uw, s.cb);
+    const float mass1 = m0 - s.F.s;
+    return s.z >= P.z_min && s.z <= P.z_max && s.v >= P.v_min && s.v <= P.v_max && mass1 >= A.m_empty;
+}
+
 // Advances one flying aircraft (not stopped before step k) by step k
 // (Sec. 3.3-3.4): control limits on the step-k values, explicit Euler step of
 // Eq. (hor) under wind and turbulence, unary limits and (arrivals) the landing
@@ -296,43 +369,9 @@ __device__ __forceinline__ bool ac_step(const ProblemC &P, const AircraftC &A, A
                                         Visit &visit, const float *pwk = nullptr)
 {
     const float dt = P.dt;
-    if (k >= s.knext) {
-        // segment s covers the steps [ceil(s H / S), ceil((s + 1) H / S)) (every
-        // segment has a step: S <= H); knext = ceil((seg + 1) H / S) advances by
-        // H = seg_q S + seg_r with its remainder carried, so no division (a late
-        // entrant passes several segments at its first step)
-        do {
-            ++s.seg;
-            s.knext += P.seg_q;
-            s.srem += P.seg_r;
-            if (s.srem >= P.S) {
-                s.srem -= P.S;
-                ++s.knext;
-            }
-        } while (k >= s.knext);
-        s.ks = k;
-        s.uw = __ldg(ul + 3 * s.seg);
-        s.uh = __ldg(ul + 3 * s.seg + 1);
-        s.ua = __ldg(ul + 3 * s.seg + 2);
-        s.zb = s.z;
-        s.vb = s.v;
-        s.cb = s.chi;
-    }
-    const float mass = m0 - s.F.s;
-    // control-derived quantities and their limits (Sec. 3.4)
-    const float sg = __fdividef(s.uh, s.v);
-    bool ok = fabsf(sg) <= P.sgmax;
-    const float cg = sqrtf(fmaxf(1.0f - sg * sg, 0.0f));
-    const float tp = __fdividef(s.uw * s.v, kG0 * cg);
-    ok = ok && (fabsf(tp) < P.tpmax);
-    const float secphi = sqrtf(fmaf(tp, tp, 1.0f));
-    const float rho = 1.225f * ex2_approx(4.2559f * __log2f(fmaxf(fmaf(-2.2558e-5f, s.z, 1.0f), 1e-30f)));
-    const float qS = A.halfS * rho * s.v * s.v;
-    const float CL = __fdividef(mass * kG0 * cg * secphi, qS);
-    const float D = qS * fmaf(A.CD2, CL * CL, A.CD0);
-    const float T = fmaf(mass, fmaf(kG0, sg, s.ua), D);
-    ok = ok && (T >= A.Tmin) && (T <= A.Tmax);
-    if (!ok) {
+    segment_advance(P, s, ul, k);
+    float cg, T;
+    if (!control_limits(P, A, s, m0, cg, T)) {
         s.dead = true;
         return false;
     }
@@ -350,25 +389,13 @@ __device__ __forceinline__ bool ac_step(const ProblemC &P, const AircraftC &A, A
     }
     w.x = fmaf(P.turb_sigma, n.x, w.x);
     w.y = fmaf(P.turb_sigma, n.y, w.y);
-    // explicit Euler step of Eq. (hor); v sin(gamma) = hdot, the speed equation
-    // reduces to v += dt a and the heading equation to chi += dt w (coordinated
-    // turn).  Within a control segment z, v and chi are linear in time: they are
-    // evaluated from the segment's start values so that rounding does not
-    // accumulate.
+    // explicit Euler step of Eq. (hor)
     float sc, cc;
     sincos_reduced(s.chi, &sc, &cc);
     const float vh = s.v * cg;
     s.x = fmaf(dt, fmaf(vh, cc, w.x), s.x);
     s.y = fmaf(dt, fmaf(vh, sc, w.y), s.y);
-    const float nk = (float)(k + 1 - s.ks) * dt;
-    s.z = fmaf(nk, s.uh, s.zb);
-    const float eta = A.Cf1 * fmaf(s.v, A.invCf2, 1.0f);
-    s.F.add(dt * eta * T);
-    s.v = fmaf(nk, s.ua, s.vb);
-    s.chi = fmaf(nk, s.uw, s.cb);
-    const float mass1 = m0 - s.F.s;
-    if (!(s.z >= P.z_min && s.z <= P.z_max && s.v >= P.v_min && s.v <= P.v_max &&
-          mass1 >= A.m_empty)) {
+    if (!air_advance(P, A, s, m0, k, T)) {
         s.dead = true;
     } else {
         s.th = atan2_poly(s.y, s.x);

@@ -14,9 +14,10 @@ namespace tma {
 
 constexpr int kMaxN = TMA_MAX_AIRCRAFT;
 constexpr int kTileParticles = 32;   // particles per rollout tile (one warp per aircraft)
-constexpr int kPairVariantBase = 8;  // first rollout variant index of the two-sample kernel
+constexpr int kPairVariantBase = 8;  // first of the five older names of the two-kernel rollout
 constexpr int kHalfVariantBase = 13; // first rollout variant index of the 16-particle (half) tile
 constexpr int kQuarterVariantBase = 16; // first rollout variant index of the 8-particle tile
+constexpr int kTrajVariantBase = 18; // first rollout variant index of the two-kernel rollout
 constexpr int kMaxRolloutVariants = 24;
 
 // Packed wind field of one (sample, step) as the rollouts read it: a float4 per
@@ -61,6 +62,7 @@ struct ProblemC {
     int grid[3];
     float dt;
     float box_lo[3], box_hi[3], inv_h[3];
+    float cell_cap[3];     // 2^23 + grid - 2: the last cell's index, as grid_cell forms it
     float turb_sigma;
     float sgmax, tpmax;    // sin(gamma_max), tan(phi_max)
     float climb_step;      // vmax sin(gamma_max) dt: largest altitude change per step
@@ -145,19 +147,22 @@ cudaError_t launch_wind_gemm(const WindC &w, const float *Lxy_t, int lda, const 
 
 cudaError_t launch_rollout(const ProblemC &P, const DynState *dyn, const float *u, const float *W,
                            int64_t L, int J, float *cost_ms, float *cost_ms_soft,
-                           unsigned long long *live, cudaStream_t st, int variant);
-// Launch-bound variants of the rollout kernel valid for the problem (indices
-// into the variant table: 0-7 the one-sample kernel, kPairVariantBase + v the
-// two-sample kernel of rollout_pair.cu, kHalfVariantBase + v and
-// kQuarterVariantBase + v the one-sample kernel on 16- and 8-particle tiles);
-// returns their number (at least 1, at most kMaxRolloutVariants).
-int rollout_variants(const ProblemC &P, int *out);
-// The two-sample kernel (shared wind field, no rolling window, M >= 2): its
-// variants valid for the problem (0-based) and its launcher.
-int rollout_pair_variants(const ProblemC &P, int *out);
-cudaError_t launch_rollout_pair(const ProblemC &P, const DynState *dyn, const float *u, const float *W,
-                                int64_t L, int J, float *cost_ms, float *cost_ms_soft,
-                                unsigned long long *live, cudaStream_t st, int variant);
+                           unsigned long long *live, cudaStream_t st, int variant, void *ws, size_t ws_bytes);
+// Variants of the rollout valid for the problem and a trajectory workspace of
+// ws_bytes (0: none): 0-7 the one-sample kernel, kHalfVariantBase + v and
+// kQuarterVariantBase + v the one-sample kernel on 16- and 8-particle tiles,
+// kTrajVariantBase + v the two-kernel rollout of rollout_traj.cu, kPairVariantBase
+// + v the same under older names; returns their number (at least 1, at most
+// kMaxRolloutVariants).  The first n_timed are the ones the autotuner times.
+int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed = nullptr);
+// The two-kernel rollout: the workspace it wants (bytes, at most 512 MB: larger
+// particle counts run in slabs; 0 when the horizon is too long for it), its
+// variants (0-based) and its launcher.
+size_t traj_workspace(const ProblemC &P, int64_t L);
+int rollout_traj_variants(const ProblemC &P, size_t ws_bytes, int *out);
+cudaError_t launch_rollout_traj(const ProblemC &P, const DynState *dyn, const float *u, const float *W, int64_t L,
+                                int J, float *cost_ms, float *cost_ms_soft, unsigned long long *live,
+                                cudaStream_t st, int variant, void *ws, size_t ws_bytes);
 cudaError_t launch_sample_mean(const float *cost_ms, int64_t L, int M, int N, float *cbar,
                                cudaStream_t st);
 
@@ -275,6 +280,8 @@ struct tma_solver {
     float *d_popdense = nullptr;          // population density cells (ProblemC::popcell), or nullptr
     void *d_work = nullptr;             // LSE workspace, then the resampling's at lse_work_bytes
     size_t work_bytes = 0, lse_work_bytes = 0;
+    void *d_traj = nullptr;             // the two-kernel rollout's trajectories (rollout_traj.cu), or nullptr
+    size_t traj_bytes = 0;
     int64_t *d_best = nullptr;
     double *d_best_sum = nullptr;
     int32_t *d_ninf = nullptr;
@@ -368,6 +375,8 @@ struct tma_batch {
     float dispatch_ms[2] = {0.f, 0.f};
     std::vector<tma::ProblemC> pc_h;    // every scenario's kernel problem (host copy)
     std::vector<int> scen_variant;      // its variant of the single-scenario rollout kernel
+    void *d_traj = nullptr;             // a trajectory workspace of traj_bytes per auxiliary stream, or nullptr
+    size_t traj_bytes = 0;
     // form 1 spreads the per-scenario launches over these streams (forked from
     // and joined to the caller's stream by events, also inside a capture)
     static constexpr int kAuxStreams = 4;
