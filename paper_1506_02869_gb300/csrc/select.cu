@@ -47,21 +47,95 @@ __device__ Cand block_best(Cand c)
     return Cand{sn[0], ss[0], sl[0]};
 }
 
+// A particle's infeasible aircraft and, in FP32, an interval that holds its FP64
+// sum: |s - S| <= N 2^-23 sum |c| covers N roundings of 2^-24 in either order and
+// those of the bound itself; an overflowing FP32 sum gives an interval that
+// excludes nothing.
+struct Bound {
+    int ninf;
+    float lo, hi;
+};
+
+__device__ __forceinline__ Bound bound_of(const float *__restrict__ c, int N, long long L)
+{
+    Bound b{0, 0.0f, 0.0f};
+    float s = 0.0f, a = 0.0f;
+#pragma unroll 8
+    for (int i = 0; i < N; ++i) {
+        const float v = __ldg(c + (size_t)i * L);
+        const bool bad = !(fabsf(v) < __int_as_float(0x7f800000));     // infinite or NaN
+        b.ninf += bad;
+        s += bad ? 0.0f : v;
+        a += bad ? 0.0f : fabsf(v);
+    }
+    const float e = (float)N * 1.1920929e-7f * a + 4.7019774e-38f * (float)N;   // and flushed subnormals
+    const bool finite = a < 1e38f;
+    b.lo = finite ? s - e : -__int_as_float(0x7f800000);
+    b.hi = finite ? s + e : __int_as_float(0x7f800000);
+    return b;
+}
+
+constexpr int kSelPer = 4;   // particles a thread looks at between two block reductions
+
+// Per-block candidates.  FP64 additions run at 2 per SM and cycle here, so summing
+// every particle in FP64 was the whole time (34 us on 24 x 262144): the particles
+// whose FP32 interval lies above another's with no more infeasible aircraft cannot
+// be chosen, and only the rest are summed in FP64 (34 -> 13 us; the 25 MB of costs
+// take 4 us to read).
 __global__ void __launch_bounds__(256) select_partial(const float *__restrict__ cbar, int N,
                                                       long long L, Cand *__restrict__ part)
 {
+    __shared__ int wn[8];
+    __shared__ float wh[8];
     Cand best{1 << 30, 0.0, 1ll << 62};
-    for (long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x; l < L;
-         l += (long long)gridDim.x * blockDim.x) {
-        int ni = 0;
-        double sum = 0.0;
-        for (int i = 0; i < N; ++i) {
-            const float c = __ldg(cbar + (size_t)i * L + l);
-            if (isinf(c) || isnan(c)) ++ni;
-            else sum += (double)c;
+    int bn = 1 << 30;                                  // least infeasible count of the block so far,
+    float bh = __int_as_float(0x7f800000);             // least upper end among those
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long l0 = (long long)blockIdx.x * blockDim.x; l0 < L; l0 += stride * kSelPer) {
+        Bound b[kSelPer];
+#pragma unroll
+        for (int q = 0; q < kSelPer; ++q) {
+            const long long l = l0 + threadIdx.x + q * stride;
+            b[q].ninf = 1 << 30;
+            if (l < L) {
+                b[q] = bound_of(cbar + l, N, L);
+                if (b[q].ninf < bn) {
+                    bn = b[q].ninf;
+                    bh = b[q].hi;
+                } else if (b[q].ninf == bn) {
+                    bh = fminf(bh, b[q].hi);
+                }
+            }
         }
-        const Cand c{ni, sum, l};
-        if (better(c, best)) best = c;
+        const int n = __reduce_min_sync(0xffffffffu, bn);
+        float h = bn == n ? bh : __int_as_float(0x7f800000);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) h = fminf(h, __shfl_xor_sync(0xffffffffu, h, o));
+        __syncthreads();                               // the previous round's values are read
+        if ((threadIdx.x & 31) == 0) {
+            wn[threadIdx.x >> 5] = n;
+            wh[threadIdx.x >> 5] = h;
+        }
+        __syncthreads();
+        bn = wn[0];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) bn = min(bn, wn[w]);
+        bh = __int_as_float(0x7f800000);
+#pragma unroll
+        for (int w = 0; w < 8; ++w)
+            if (wn[w] == bn) bh = fminf(bh, wh[w]);
+#pragma unroll
+        for (int q = 0; q < kSelPer; ++q) {
+            const long long l = l0 + threadIdx.x + q * stride;
+            if (l >= L || b[q].ninf != bn || !(b[q].lo <= bh)) continue;
+            double sum = 0.0;
+            for (int i = 0; i < N; ++i) {
+                const float c = __ldg(cbar + (size_t)i * L + l);
+                if (!(isinf(c) || isnan(c))) sum += (double)c;
+            }
+            const Cand c{b[q].ninf, sum, l};
+            if (better(c, best)) best = c;
+        }
     }
     best = block_best(best);
     if (threadIdx.x == 0) part[blockIdx.x] = best;
