@@ -51,7 +51,9 @@ __host__ __device__ constexpr int wind_tile_cols(int T, int nz)
 
 // C[p][col] = sum_{q <= p} At[q][p] Btmp[q][col], q ascending in one chain of
 // fused multiply-adds per output, sigma C into the packed layout.  T x T tiles,
-// 8 x 8 outputs per thread (T = 128: 256 threads, T = 64: 64), K in steps of 8
+// T = 64, 8 x 8 outputs per thread (64 threads: the two warps of a block wait for
+// little, and small fields fill the chip; 128 x 128 tiles of 256 threads were 8-30 %
+// slower from 5 samples of a 32 x 32 x 8 grid over 90 steps on), K in steps of 8
 // through a ring of four stages filled by cp.async; a pair of columns per
 // two-lane FP32 instruction (each lane the IEEE single operation), which halves
 // the issue slots of the products.  At is the factor transposed and zero-padded
@@ -59,13 +61,13 @@ __host__ __device__ constexpr int wind_tile_cols(int T, int nz)
 // guards for the last columns only.  Row tiles run from the last (longest sums)
 // to the first.  Bound: the FP32 units (2.6e11 products and sums for 16 samples of
 // a 64 x 64 x 8 grid over 60 steps, 3.2 ms at their peak): that field with its
-// plain values takes 4.57 ms (normals included) against 9.47 ms with a
+// plain values takes 4.18 ms (normals included) against 9.47 ms with a
 // single-buffered loop, a second pass that formed the differences and a strided
 // copy for the plain values.
 constexpr int kStages = 4, kKStep = 8;
 
 template <int T>
-__global__ void __launch_bounds__(T *T / 64, T == 128 ? 2 : 6)
+__global__ void __launch_bounds__(T *T / 64, 6)
     wind_gemm_kernel(const WindC w, const float *__restrict__ At, int lda, const float *__restrict__ Bm, int n_ctiles,
                      int n_rtiles, float4 *__restrict__ W, float2 *__restrict__ Wown)
 {
@@ -190,22 +192,11 @@ cudaError_t launch_wind_normals_ar(const WindC &w, const DynState *dyn, float *B
 cudaError_t launch_wind_gemm(const WindC &w, const float *Lxy_t, int lda, const float *Btmp,
                              float *W, cudaStream_t st, float *W_own)
 {
-    const auto tiles = [&](int T, int &ct, int &rt) {
-        const int cols = wind_tile_cols(T, w.nz);
-        ct = (w.ncol + cols - 1) / cols;
-        rt = (w.nxy + T - 1) / T;
-    };
-    int ct, rt;
-    tiles(128, ct, rt);
-    float4 *W4 = reinterpret_cast<float4 *>(W);
-    float2 *W2 = reinterpret_cast<float2 *>(W_own);
-    // fewer 128 x 128 tiles than two per SM: 64 x 64 tiles keep the chip busier
-    if ((long long)ct * rt >= 2 * 152) {
-        wind_gemm_kernel<128><<<ct * rt, 256, 0, st>>>(w, Lxy_t, lda, Btmp, ct, rt, W4, W2);
-    } else {
-        tiles(64, ct, rt);
-        wind_gemm_kernel<64><<<ct * rt, 64, 0, st>>>(w, Lxy_t, lda, Btmp, ct, rt, W4, W2);
-    }
+    constexpr int T = 64;
+    const int cols = wind_tile_cols(T, w.nz);
+    const int ct = (w.ncol + cols - 1) / cols, rt = (w.nxy + T - 1) / T;
+    wind_gemm_kernel<T><<<ct * rt, T * T / 64, 0, st>>>(w, Lxy_t, lda, Btmp, ct, rt, reinterpret_cast<float4 *>(W),
+                                                       reinterpret_cast<float2 *>(W_own));
     count_launch();
     return cudaGetLastError();
 }
