@@ -103,16 +103,19 @@ int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed)
         return false;
     };
     // With the two-kernel form at hand the one-sample kernel is the faster one
-    // only for small work (2 aircraft, 1024 particles, 8 samples: 23 against 33 us),
-    // where its register budget decides: one variant of each is timed.
+    // only for small work (2 aircraft, 1024 particles, 8 samples: 23 against 33 us;
+    // 32 aircraft, 200 particles, 8 samples: 196 on half tiles, 262 on whole ones),
+    // where its register budget and tile decide: one variant of each is timed.
     for (int c = 0; c < nt; ++c) out[n++] = kTrajVariantBase + tv[c];
     for (int v : {3, 7, 4})                      // 128, 85 and 64 registers
         if (nt > 0 && fits(v)) out[n++] = v;
+    if (nt > 0 && small_tile_valid(P, 16, kHalfVariants[0].max_threads)) out[n++] = kHalfVariantBase;
     if (n_timed && nt > 0) *n_timed = n;
     for (int v = 0; v < kNumVariants; ++v)
         if (fits(v) && !listed(v)) out[n++] = v;
     for (int v = 0; v < kNumHalfVariants; ++v)
-        if (small_tile_valid(P, 16, kHalfVariants[v].max_threads)) out[n++] = kHalfVariantBase + v;
+        if (small_tile_valid(P, 16, kHalfVariants[v].max_threads) && !listed(kHalfVariantBase + v))
+            out[n++] = kHalfVariantBase + v;
     for (int v = 0; v < kNumQuarterVariants; ++v)
         if (small_tile_valid(P, 8, kQuarterVariants[v].max_threads)) out[n++] = kQuarterVariantBase + v;
     if (n_timed && nt == 0) *n_timed = n;
