@@ -3,73 +3,36 @@
 // and Sec. 7.1 with the softplus separation penalty; unary and control limits
 // stay hard) for every particle l, used by the Langevin move.
 //
-// Mapping: as the rollout, one block is 32 particles (lanes) x N aircraft
-// (warps); a block takes a contiguous range of wind samples.  For each sample:
-//   pass 1  the forward rollout of each aircraft alone (the step function of
-//           the rollout kernel), saving a checkpoint of the aircraft state
-//           every 10 steps; its J_T fixes the cost coefficients of the
-//           reverse sweep.  No exchange between aircraft is needed yet;
-//   pass 2  for each checkpoint interval, last to first: recompute its steps
-//           from the checkpoint, keeping the pre-step states and the
-//           derivative of the per-step cost terms at the post-step state
-//           (deviation terms, and the separation penalty with its value, the
-//           partner positions coming through a shared-memory exchange as in
-//           the rollout); then run the interval's steps backwards, carrying
-//           the adjoint (x, y, z, v, chi, F) of this aircraft and summing the
-//           control gradient of each segment.
+// The wind enters the position alone, so the adjoint splits as the rollout does
+// (rollout_traj.cu).  The adjoints of x and y run backwards under each sample; those of
+// altitude, airspeed, heading and fuel propagate through factors that no sample
+// changes, and they are linear in what x and y feed them, so they run once on the
+// sums over the samples:
+//   trajectory_kernel     the wind-independent records, once per particle;
+//   grad_samples_kernel   per sample: the forward pass of the rollout, keeping the
+//                         positions and the penalties' derivatives; its J_T fixes the
+//                         cost coefficients; then backwards with the adjoint (x, y),
+//                         adding the step's x and y adjoints and what they and the
+//                         cost terms feed the altitude and the heading to sums over
+//                         the block's samples (a block takes 32, 16 or 8 particles and a
+//                         range of the samples, one after the other: no atomics, a
+//                         fixed order);
+//   grad_controls_kernel  the costs' means over the samples; once per particle:
+//                         backwards with the summed sources, the altitude, airspeed, heading
+//                         and fuel adjoints, and each segment's control gradient.
 // Limit, landing and interpolation-cell decisions keep their forward values.
-// Once the forward pass is stored, the reverse sweep needs nothing from the
-// other aircraft: the separation derivative with respect to this aircraft's
-// position depends only on forward positions.
-#include "rollout_tile.cuh"
+//
+// Bound: instruction issue (54 % busy, 780 warp instructions a step of 32 aircraft,
+// forward and back together; 1400 with the whole adjoint per sample) and the latency
+// of the wind gathers, here twice a step; DRAM 28 % for the sums and the flight log.
+// Late particles, 12 aircraft, L 16384, M 16: 11.5 -> 7.3 ms; 24 aircraft, L 4096, M 8,
+// 90 steps: 6.05 -> 3.64 ms; 6 aircraft, L 4096, M 8: 0.67 -> 0.58 ms.  Of the 7.3 ms
+// the backward half is 3.2, the pairs 1.5, grad_controls_kernel 0.2.
+#include "wind_rollout.cuh"
 
 namespace tma {
 
 namespace {
-
-constexpr int kCkEvery = 10;
-constexpr int kMaxCk = TMA_MAX_GRAD_HORIZON / kCkEvery;
-
-struct Checkpoint {
-    float x, y, z, v, chi, Fs, Fc, zb, vb, cb;
-    int ks, segflags;     // segment + 1 in bits 0..19, dead bit 20, landed bit 21
-};
-
-__device__ __forceinline__ Checkpoint save(const AcState &s)
-{
-    Checkpoint c;
-    c.x = s.x; c.y = s.y; c.z = s.z; c.v = s.v; c.chi = s.chi;
-    c.Fs = s.F.s; c.Fc = s.F.c;
-    c.zb = s.zb; c.vb = s.vb; c.cb = s.cb;
-    c.ks = s.ks;
-    c.segflags = (s.seg + 1) | (s.dead ? 1 << 20 : 0) | (s.landed ? 1 << 21 : 0);
-    return c;
-}
-
-__device__ __forceinline__ void restore(const ProblemC &P, AcState &s, const Checkpoint &c,
-                                        const float *__restrict__ ul)
-{
-    s.x = c.x; s.y = c.y; s.z = c.z; s.v = c.v; s.chi = c.chi;
-    s.F.s = c.Fs; s.F.c = c.Fc;
-    s.zb = c.zb; s.vb = c.vb; s.cb = c.cb;
-    s.ks = c.ks;
-    s.seg = (c.segflags & 0xFFFFF) - 1;
-    s.dead = (c.segflags >> 20) & 1;
-    s.landed = (c.segflags >> 21) & 1;
-    if (s.seg >= 0) {
-        const long long B = (long long)(s.seg + 1) * P.H + P.S - 1;
-        s.knext = (int)(B / P.S);
-        s.srem = (int)(B % P.S);
-        s.uw = __ldg(ul + 3 * s.seg);
-        s.uh = __ldg(ul + 3 * s.seg + 1);
-        s.ua = __ldg(ul + 3 * s.seg + 2);
-    } else {
-        s.knext = 0;
-        s.srem = P.S - 1;
-    }
-}
-
-__device__ __forceinline__ float sgnf(float a) { return a > 0.0f ? 1.0f : (a < 0.0f ? -1.0f : 0.0f); }
 
 // wrapped angle in [-pi, pi] (the signed counterpart of angdist)
 __device__ __forceinline__ float wrapf(float a)
@@ -161,86 +124,214 @@ __device__ __forceinline__ CostGrad cost_grad(const ProblemC &P, const AircraftC
     return g;
 }
 
-// Derivative of this aircraft's per-step deviation terms at a flying
-// step-(k+1) state, as a step visitor: the sources (x, y, z, v, chi) that enter
-// the adjoint at step k+1.
-struct TermGrad {
-    CostGrad cg;
-    float sx = 0.f, sy = 0.f, sz = 0.f, sv = 0.f, sc = 0.f;
 
-    __device__ __forceinline__ void bearing(const AcState &s, float coef)
+// Derivative of a pair of deviation terms with respect to the position a sample
+// reaches at a step: (x, y) go to the sample's own adjoint, z and chi to the sums.
+struct Sources {
+    float x = 0.f, y = 0.f, z = 0.f, chi = 0.f;
+    __device__ __forceinline__ void bearing(float px, float py, float coef)
     {
-        const float r2 = fmaf(s.x, s.x, s.y * s.y);
+        const float r2 = fmaf(px, px, py * py);
         const float ir2 = r2 > 0.0f ? 1.0f / r2 : 0.0f;
-        sx = fmaf(coef, -s.y * ir2, sx);
-        sy = fmaf(coef, s.x * ir2, sy);
+        x = fmaf(coef, -py * ir2, x);
+        y = fmaf(coef, px * ir2, y);
     }
-    __device__ __forceinline__ void departure(const ProblemC &P, const AircraftC &A, const AcState &s)
+    // th, beta: the bearing and the glide angle there
+    __device__ __forceinline__ void arrival(const ProblemC &P, const CostGrad &cg, float px, float py, float pz, float chi1,
+                                            float th, float beta)
     {
-        bearing(s, sgnf(wrapf(s.th - A.thF)) * cg.gA);
-        sz = fmaf(cg.gB, sgnf(s.z - A.Z), sz);
-        sv = fmaf(cg.gC, sgnf(s.v - A.vD), sv);
-    }
-    __device__ __forceinline__ void arrival(const ProblemC &P, const AircraftC &A, const AcState &s)
-    {
-        const float se = sgnf(wrapf(s.chi - fmaf(2.0f, s.th, kPi))) * cg.gA;
-        sc += se;
-        bearing(s, -2.0f * se);
+        const float se = sgnf(wrapf(chi1 - fmaf(2.0f, th, kPi))) * cg.gA;
+        chi += se;
+        bearing(px, py, -2.0f * se);
         // glide angle beta = atan2(z, r ratio(theta)), ratio = |theta| / sin|theta|
-        const float x = s.x, y = s.y, z = s.z;
-        const float r2 = fmaf(x, x, y * y);
-        const float r = sqrtf(r2);
-        const float ath = fabsf(s.th);
+        const float r = sqrtf(fmaf(px, px, py * py));
+        const float ath = fabsf(th);
         float ratio, dratio;
         if (ath < 1e-3f) {
-            ratio = fmaf(s.th * s.th, 1.0f / 6.0f, 1.0f);
-            dratio = s.th * (1.0f / 3.0f);
+            ratio = fmaf(th * th, 1.0f / 6.0f, 1.0f);
+            dratio = th * (1.0f / 3.0f);
         } else {
             float sn, cs;
             __sincosf(ath, &sn, &cs);                 // ath in [0, pi]: no range reduction needed
             if (sn >= 0.25f * ath) {
                 ratio = ath / sn;
-                dratio = sgnf(s.th) * (sn - ath * cs) / (sn * sn);
+                dratio = sgnf(th) * (sn - ath * cs) / (sn * sn);
             } else {
                 ratio = 4.0f;
                 dratio = 0.0f;
             }
         }
         const float sa = r * ratio;
-        const float den = fmaf(z, z, sa * sa);
-        const float bb = cg.gB * sgnf(s.beta - P.beta_f);
-        sz = fmaf(bb, sa / den, sz);
+        const float den = fmaf(pz, pz, sa * sa);
+        const float bb = cg.gB * sgnf(beta - P.beta_f);
+        z = fmaf(bb, sa / den, z);
         // d(sa)/dx = ratio x / r + r ratio'(theta) dtheta/dx, likewise for y
-        const float bsa = -bb * z / den;
+        const float bsa = -bb * pz / den;
         const float ir = r > 0.0f ? 1.0f / r : 0.0f;
-        sx = fmaf(bsa, ratio * x * ir, sx);
-        sy = fmaf(bsa, ratio * y * ir, sy);
-        bearing(s, bsa * r * dratio);
+        x = fmaf(bsa, ratio * px * ir, x);
+        y = fmaf(bsa, ratio * py * ir, y);
+        bearing(px, py, bsa * r * dratio);
     }
-    __device__ __forceinline__ void noise(const ProblemC &P, const AircraftC &A, const AcState &s)
+    __device__ __forceinline__ void noise(const ProblemC &P, const CostGrad &cg, float px, float py, float pz)
     {
-        float gx, gy;
-        const float pd = popdense_grad(P, s.x, s.y, gx, gy);
-        const float za = s.z * P.Ac_inv;
+        const float za = pz * P.Ac_inv;
         const float h = fmaf(-za, za, 1.0f);
         if (h > 0.0f) {
-            sx = fmaf(cg.gN * h, gx, sx);
-            sy = fmaf(cg.gN * h, gy, sy);
-            sz = fmaf(cg.gN * pd, -2.0f * s.z * P.Ac_inv * P.Ac_inv, sz);
+            float gx, gy;
+            const float pd = popdense_grad(P, px, py, gx, gy);
+            x = fmaf(cg.gN * h, gx, x);
+            y = fmaf(cg.gN * h, gy, y);
+            z = fmaf(cg.gN * pd, -2.0f * pz * P.Ac_inv * P.Ac_inv, z);
         }
     }
 };
 
-// Adjoint of step k of one aircraft (Eq. (hor) with the drag of the
-// coordinated turn in closed form, D = q CD0 + CD2 m^2 (g^2 cos^2(gamma) +
-// w^2 v^2) / q, q = rho v^2 S / 2): maps the adjoint at k+1 to the adjoint at
-// k and adds the step's control derivative to (gw, gh, ga).
-__device__ __forceinline__ void step_adjoint(const ProblemC &P, const AircraftC &A,
-                                             const float4 *__restrict__ Wk, float x, float y,
-                                             float z, float v, float chi, float mass, float uw,
-                                             float uh, float ua, float &X, float &Y, float &Z,
-                                             float &V, float &CH, float &FF, float &gw, float &gh,
-                                             float &ga)
+// Scratch of a slab of n particles and nchunk ranges of samples, in the records' tiles;
+// element ((g H + k) B + t) with g = range n_tiles + tile.
+struct GradScratch {
+    FlightLog log;     // the current sample's flight
+    float4 *acc;       // sums over the range's samples: adjoints of x and y after step k; what feeds those of z and chi there
+    float *land;       // fuel coefficients of the samples that landed at step k (arrivals)
+    float4 *sums;      // [g][B]: sums of the samples' coefficients of altitude, speed and (not landed) fuel
+};
+
+template <int kMinBlocks, int TP>
+__global__ void __launch_bounds__(256, kMinBlocks)
+    grad_samples_kernel(const ProblemC P, const DynState *__restrict__ dyn, const float4 *__restrict__ W, const TrajOut R,
+                        const GradScratch G, long long L, long long l_begin, long long l_end, int n_tiles, int m_per_block,
+                        int J, float *__restrict__ cost_ms)
+{
+    extern __shared__ __align__(16) float sh[];
+    grid_begin();
+    const int N = P.N, H = P.H, B = N * TP;
+    const int t = threadIdx.x, i = t / TP, j = t % TP;
+    const int range = blockIdx.x / n_tiles, tile = blockIdx.x - range * n_tiles;
+    const long long l = l_begin + (long long)tile * TP + j;
+    const bool exists = l < l_end;
+    const uint32_t mpc = dyn->mpc_step;
+    const int type = P.ac[i].type;
+    const float target = type == 0 ? P.beta_f : P.ac[i].thF;
+    const int kd = __float_as_int(R.fin[(size_t)tile * B + t].w);
+    const float invM = 1.0f / (float)P.M;
+    const float sep_c = 2.0f * P.mu_sep * invM;        // each pair enters two aircraft's costs
+    const unsigned g0 = (unsigned)blockIdx.x * H * B + t;         // the scratch bound keeps these within 32 bits
+    const unsigned r0 = (unsigned)tile * H * B + t;
+    float sB = 0.0f, sC = 0.0f, sF = 0.0f;
+    float sinF, cosF;
+    sincosf(P.ac[i].thF, &sinF, &cosF);
+    if (type == 0)
+        for (int k = 0; k < H; ++k) G.land[g0 + (unsigned)k * B] = 0.0f;
+    const int mb = range * m_per_block, me = min(P.M, mb + m_per_block);
+    for (int m = mb; m < me; ++m) {
+        if (m > mb) __syncthreads();              // the previous sample's positions are read
+        const float4 *Wm = W + (size_t)m * H * P.P;
+        const Flown q = wind_forward<TP, false, true, true>(P, dyn, Wm, R, sh, tile, t, l, m, J, mpc, type, target, 0, kd,
+                                                            G.log, (int)blockIdx.x, sep_c);
+        const bool dead = !q.landed && kd < H;
+        CostGrad cg;
+        {
+            const AircraftC A = P.ac[i];
+            const float4 fn = R.fin[(size_t)tile * B + t];
+            const AltBounds ab = alt_bounds(P, A, dyn->x0[i][2], H);
+            CostSums cs;
+            cs.sA = q.sA;
+            cs.sB = q.sB;
+            if (type != 0) {
+                cs.sB.s = fn.x;
+                cs.sC.s = fn.y;
+            }
+            cs.sN = q.sN;
+            const float Fs = q.landed ? __ldg(R.fuel + r0 + (unsigned)(q.k_end - 1) * B) : fn.z;
+            const float JT = total_objective(P, A, cs, Fs, ab, H);
+            if (exists)
+                cost_ms[((size_t)m * N + i) * (size_t)L + l] =
+                    dead ? __int_as_float(0x7f800000) : fmaf(P.mu_sep, q.soft, -logf(fmaxf(JT, 1e-30f)));
+            cg = cost_grad(P, A, JT, ab, invM);
+        }
+        if (dead || !exists) continue;             // an infeasible particle's gradient is zero
+        // the landing step itself has no terms, only the fuel burned up to it
+        const int k_top = q.landed ? q.k_end - 1 : H;
+        if (q.landed) {
+            G.land[g0 + (unsigned)k_top * B] += cg.gF;
+        } else {
+            sF += cg.gF;
+        }
+        if (type != 0) {
+            sB += cg.gB;
+            sC += cg.gC;
+        }
+        if (m == mb)
+            for (int k = k_top; k < H; ++k) G.acc[g0 + (unsigned)k * B] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k_top == 0) continue;
+        float X = 0.0f, Y = 0.0f, zc = 0.0f;       // adjoints of the position; what step k + 1 feeds the altitude's
+        // positions after step k, before it, and before step k - 1, the last one in
+        // flight while step k is worked on (its wind cell's address needs it)
+        const float2 pi = make_float2(dyn->x0[i][0], dyn->x0[i][1]);
+        const float zi = dyn->x0[i][2];
+        unsigned o = (unsigned)(k_top - 1) * B;
+        float2 p = G.log.xy[g0 + o], p0 = pi;
+        float z = __ldg(R.air + r0 + o).x, z0 = zi;
+        if (k_top > 1) {
+            p0 = G.log.xy[g0 + o - B];
+            z0 = __ldg(R.air + r0 + o - B).x;
+        }
+        for (int k = k_top - 1; k >= 0; --k) {
+            float2 pn = pi;
+            float zn = zi;
+            if (k > 1) {
+                pn = G.log.xy[g0 + o - 2 * B];
+                zn = __ldg(R.air + r0 + o - 2 * B).x;
+            }
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (m > mb) a = G.acc[g0 + o];
+            float2 pol = make_float2(0.f, 0.f);
+            if (type == 0) pol = G.log.polar[g0 + o];
+            const unsigned near = G.log.near[((unsigned)blockIdx.x * n_chunks(H) + (unsigned)(k / kStepsPerBarrier)) * B + t];
+            float2 dwx, dwy, dwz;
+            wind_grad(P, Wm + (size_t)k * P.P, p0.x, p0.y, z0, dwx, dwy, dwz);
+            Sources s;
+            // a departure's bearing error has the sign of the cross product of its
+            // target direction and its position
+            if (type == 0) s.arrival(P, cg, p.x, p.y, z, __ldg(R.chi + r0 + o), pol.x, pol.y);
+            else s.bearing(p.x, p.y, sgnf(fmaf(cosF, p.y, -sinF * p.x)) * cg.gA);
+            if (P.w_noise != 0.0f) s.noise(P, cg, p.x, p.y, z);
+            if ((near >> (k % kStepsPerBarrier)) & 1u) {
+                const float4 d = G.log.sep[g0 + o];
+                s.x += d.x;
+                s.y += d.y;
+                s.z += d.z;
+            }
+            X += s.x;
+            Y += s.y;
+            G.acc[g0 + o] = make_float4(a.x + X, a.y + Y, a.z + (s.z + zc), a.w + s.chi);
+            const float nX = X + P.dt * fmaf(X, dwx.x, Y * dwx.y);
+            const float nY = Y + P.dt * fmaf(X, dwy.x, Y * dwy.y);
+            zc = P.dt * fmaf(X, dwz.x, Y * dwz.y);
+            X = nX;
+            Y = nY;
+            p = p0;
+            z = z0;
+            p0 = pn;
+            z0 = zn;
+            o -= B;
+        }
+    }
+    G.sums[(size_t)blockIdx.x * B + t] = make_float4(sB, sC, sF, 0.0f);
+}
+
+// Derivatives of step k of one aircraft that no sample changes (Eq. (hor) with the
+// drag of the coordinated turn in closed form, D = q CD0 + CD2 m^2 (g^2 cos^2(gamma)
+// + w^2 v^2) / q, q = rho v^2 S / 2), times the step dt where they enter.
+struct StepCoef {
+    float cc, sc;              // heading
+    float vP, cP, hP;          // along-track adjoint to V, cross-track to CH, along-track to the climb control
+    float e;                   // fuel adjoint to the thrust: dt eta
+    float zT, vT, mT;          // thrust (fuel) to Z, V (with eta's own share), and to FF
+    float wT, hT, aT;          // thrust to the controls
+};
+
+__device__ __forceinline__ StepCoef step_coef(const ProblemC &P, const AircraftC &A, float z, float v, float chi,
+                                              float mass, float uw, float uh, float ua)
 {
     const float dt = P.dt;
     const float iv = 1.0f / v;
@@ -267,390 +358,264 @@ __device__ __forceinline__ void step_adjoint(const ProblemC &P, const AircraftC 
     const float dD_dz = fmaf(A.CD0, dq_dz, -K2 * A2 * dq_dz * iq * iq);
     const float dD_dm = 2.0f * A.CD2 * mass * A2 * iq;
     const float dT_dv = fmaf(-mass * kG0 * uh, iv * iv, dD_dv);
-    const float dT_dm = ua + kG0 * sg + dD_dm;
-    const float dT_dh = fmaf(mass * kG0, iv, K2 * dA2_dh * iq);
-    const float dT_dw = K2 * dA2_dw * iq;
     const float eta = A.Cf1 * fmaf(v, A.invCf2, 1.0f);
     const float deta_dv = A.Cf1 * A.invCf2;
-    float2 dwx, dwy, dwz;
-    wind_grad(P, Wk, x, y, z, dwx, dwy, dwz);
-    float sc, cc;
-    sincos_reduced(chi, &sc, &cc);
-    const float proj = fmaf(cc, X, sc * Y);            // along-track adjoint
-    const float fe = FF * dt * eta;                     // fuel adjoint times d F'/d T
-    const float nX = X + dt * fmaf(X, dwx.x, Y * dwx.y);
-    const float nY = Y + dt * fmaf(X, dwy.x, Y * dwy.y);
-    const float nZ = Z + dt * fmaf(X, dwz.x, Y * dwz.y) + fe * dD_dz;
-    const float nV = V + dt * (cg + v * dcg_dv) * proj + FF * dt * fmaf(deta_dv, T, eta * dT_dv);
-    const float nC = CH + dt * v * cg * fmaf(-sc, X, cc * Y);
-    const float nF = FF - fe * dT_dm;
-    gw += fmaf(dt, CH, fe * dT_dw);
-    gh += dt * Z + dt * v * dcg_dh * proj + fe * dT_dh;
-    ga += fmaf(dt, V, fe * mass);
-    X = nX; Y = nY; Z = nZ; V = nV; CH = nC; FF = nF;
+    StepCoef c;
+    sincos_reduced(chi, &c.sc, &c.cc);
+    c.vP = dt * (cg + v * dcg_dv);
+    c.cP = dt * v * cg;
+    c.hP = dt * v * dcg_dh;
+    c.e = dt * eta;
+    c.zT = dD_dz;
+    c.vT = dt * fmaf(deta_dv, T, eta * dT_dv);
+    c.mT = ua + kG0 * sg + dD_dm;
+    c.wT = K2 * dA2_dw * iq;
+    c.hT = fmaf(mass * kG0, iv, K2 * dA2_dh * iq);
+    c.aT = mass;
+    return c;
 }
 
-// Derivative of one pair's separation penalty (weight w = 2 mu sigma(beta g) / M)
-// with respect to this aircraft's position, from the differences own - partner.
-__device__ __forceinline__ void pair_grad(const ProblemC &P, float w, float dx, float dy, float dz,
-                                          float &sx, float &sy, float &sz)
+// The sums of four steps are gathered at a time, their loads in flight together.
+template <int TP>
+__global__ void __launch_bounds__(256, 2) grad_controls_kernel(const ProblemC P, const DynState *__restrict__ dyn,
+                                                            const float *__restrict__ u, const TrajOut R,
+                                                            const GradScratch G, long long l_begin, long long l_end,
+                                                            int n_tiles, int n_ranges, const float *__restrict__ cost_ms,
+                                                            long long L, float *__restrict__ cost,
+                                                            float *__restrict__ grad, float *__restrict__ cbar)
 {
-    const float dh = sqrtf(fmaf(dx, dx, dy * dy));
-    const float ghh = fmaf(-dh, P.Sh_inv, 1.0f);
-    const float gvv = fmaf(-fabsf(dz), P.Sv_inv, 1.0f);
-    if (ghh <= gvv) {
-        if (dh > 0.0f) {
-            const float eh = w * P.Sh_inv / dh;
-            sx = fmaf(-eh, dx, sx);
-            sy = fmaf(-eh, dy, sy);
-        }
-    } else {
-        sz = fmaf(-w * P.Sv_inv, sgnf(dz), sz);
-    }
-}
-
-// The penalty of a pair and the logistic weight of its derivative, from one
-// exponential of -|beta g| (0, 0 when either aircraft is not flying: its
-// published altitude is far away).
-__device__ __forceinline__ float2 pair_penalty(const ProblemC &P, float dx, float dy, float dz)
-{
-    const float dh = sqrtf(fmaf(dx, dx, dy * dy));
-    const float gmin = fminf(fmaf(-dh, P.Sh_inv, 1.0f), fmaf(-fabsf(dz), P.Sv_inv, 1.0f));
-    const float bg = P.sp_beta * gmin;
-    const float e = __expf(-fabsf(bg));
-    return make_float2((fmaxf(bg, 0.0f) + log1p_unit(e)) * P.sp_inv_beta,
-                       (bg >= 0.0f ? 1.0f : e) / (1.0f + e));
-}
-
-// Pairs are computed once (as in the rollout) when the received slots fit in
-// shared memory; above this aircraft count every aircraft computes its N-1.
-constexpr int kGradPairOnceMaxN = 16;
-
-// Positions are triple-buffered by step: a receiver reads its partners'
-// positions of step k-1 at step k, after the step-k barrier; a partner can
-// overwrite that buffer only at step k+2, after the step-(k+1) barrier, which
-// the receiver reaches after its read.
-__host__ __device__ constexpr int grad_smem_words(int N)
-{
-    return 12 * N * kTileParticles +                                              // positions
-           (N <= kGradPairOnceMaxN ? 4 * N * tile_pair_slots(N) * kTileParticles : 0);  // slots
-}
-
-template <int kMaxThreads, int kMinBlocks>
-__global__ void __launch_bounds__(kMaxThreads, kMinBlocks)
-rollout_grad_kernel(const ProblemC P, const DynState *__restrict__ dyn, const float *__restrict__ u,
-                    const float4 *__restrict__ W, long long L, int nLb, int m_per_block, int J,
-                    float *__restrict__ cost_ms, float *__restrict__ gpart)
-{
-    extern __shared__ float spos[];
-    const int N = P.N;
-    const int i = threadIdx.x >> 5, j = threadIdx.x & 31;
-    const int chunk = blockIdx.x / nLb;
-    const long long l = (long long)(blockIdx.x - chunk * nLb) * kPB + j;
-    const bool exists = l < L;
-    const AircraftC A = P.ac[i];   // a copy: the warp-uniform constants stay in registers
-    const uint32_t mpc = dyn->mpc_step;
-    const float m0 = dyn->x0[i][5];
-    const float *ul = u + ((size_t)(exists ? l : 0) * N + i) * (size_t)(P.S * 3);
-    const int nS3 = P.S * 3;
-    float *gout = gpart + (((size_t)chunk * L + (exists ? l : 0)) * N + i) * (size_t)nS3;
-    if (exists)
-        for (int n = 0; n < nS3; ++n) gout[n] = 0.0f;
-    const int plane = N * kPB;
-    // shared memory: positions float4 [3][N][32], then (pair-once) the received
-    // (penalty, logistic weight) float2 [2][N][slots][32]
-    float4 *pos = reinterpret_cast<float4 *>(spos);
-    float2 *slots = reinterpret_cast<float2 *>(spos + 12 * plane);
-    const bool pair_once = N <= kGradPairOnceMaxN;
-    const int n_slots = tile_pair_slots(N);
-    const int n_half = (N - 1) >> 1;
-    const bool even_n = (N & 1) == 0;
-    const int n_pairs = n_half + ((even_n && i < (N >> 1)) ? 1 : 0);
-    const int n_recv = n_half + ((even_n && i >= (N >> 1)) ? 1 : 0);
-    const float invM = 1.0f / (float)P.M;
-    const float sep_c = 2.0f * P.mu_sep * invM;        // each pair enters two aircraft's costs
-    const int mb = chunk * m_per_block, me = min(P.M, mb + m_per_block);
-    const int nck = (P.H + kCkEvery - 1) / kCkEvery;
-
-    Checkpoint ck[kMaxCk];
-    float hx[kCkEvery], hy[kCkEvery], hz[kCkEvery], hv[kCkEvery], hc[kCkEvery], hF[kCkEvery];
-    float rx[kCkEvery], ry[kCkEvery], rz[kCkEvery], rv[kCkEvery], rc[kCkEvery];
-
-    for (int m = mb; m < me; ++m) {
-        const float4 *Wm = W + (size_t)m * P.H * P.P;
-        // ---------------- pass 1: forward rollout of this aircraft alone, with
-        // checkpoints; J_T fixes the cost coefficients of the reverse sweep
-        AcState s;
-        ac_init(s, dyn, i, exists, P.S);
-        const AltBounds ab = alt_bounds(P, A, s.z, P.H);
-        CostSums cs;
-        for (int k = 0; k < P.H; ++k) {
-            if (k % kCkEvery == 0) ck[k / kCkEvery] = save(s);
-            if (!s.dead && !s.landed)
-                ac_step<true>(P, A, s, ul, Wm + (size_t)k * P.P, m0, (uint32_t)l, (uint32_t)i,
-                        (uint32_t)m, k, J, mpc, cs);
-        }
-        const float JT = total_objective(P, A, cs, s.F.s, ab, P.H);
-        const float c = -logf(fmaxf(JT, 1e-30f));
-        const bool dead = s.dead;
-        const CostGrad cg = cost_grad(P, A, JT, ab, invM);
-        float soft = 0.0f;     // separation penalty, summed in pass 2
-
-        // ---------------- pass 2: interval by interval, last to first
-        float X = 0.f, Y = 0.f, Z = 0.f, V = 0.f, CH = 0.f, FF = cg.gF;
-        int gseg = -1;
-        float gw = 0.f, gh = 0.f, ga = 0.f;
-        for (int c_i = nck - 1; c_i >= 0; --c_i) {
-            const int k0 = c_i * kCkEvery, k1 = min(P.H, k0 + kCkEvery);
-            AcState r;
-            ac_init(r, dyn, i, exists, P.S);
-            restore(P, r, ck[c_i], ul);
-            unsigned upd = 0;
-            // the previous interval's last exchange may still be read
-            tile_barrier(0, blockDim.x);
-            for (int k = k0; k < k1; ++k) {
-                const int t = k - k0;
-                hx[t] = r.x; hy[t] = r.y; hz[t] = r.z; hv[t] = r.v; hc[t] = r.chi; hF[t] = r.F.s;
-                TermGrad tg;
-                tg.cg = cg;
-                if (!r.dead && !r.landed &&
-                    ac_step<true>(P, A, r, ul, Wm + (size_t)k * P.P, m0, (uint32_t)l, (uint32_t)i,
-                            (uint32_t)m, k, J, mpc, tg))
-                    upd |= 1u << t;
-                const bool act = !r.dead && !r.landed;
-                float sx = tg.sx, sy = tg.sy, sz = tg.sz, sv = tg.sv, sc = tg.sc;
-                float4 *buf = pos + (k % 3) * plane;
-                buf[i * kPB + j] = make_float4(r.x, r.y, act ? r.z : 1e30f, 0.0f);
-                tile_barrier(0, blockDim.x);
-                if (pair_once) {
-                    // pairs the partners computed for this aircraft at the previous
-                    // step: penalty, and the derivative from both positions of then
-                    if (k > k0) {
-                        const float2 *rr = slots + ((((k - 1) & 1) * N + i) * n_slots) * kPB + j;
-                        const float4 *pb = pos + ((k - 1) % 3) * plane;
-                        float px = 0.f, py = 0.f, pz = 0.f;
-                        int o = i;
-                        for (int d = 0; d < n_recv; ++d) {
-                            o = (o == 0) ? N - 1 : o - 1;
-                            const float2 ps = rr[d * kPB];
-                            soft += ps.x;
-                            if (ps.y != 0.0f) {
-                                const float4 q = pb[o * kPB + j];
-                                pair_grad(P, sep_c * ps.y, hx[t] - q.x, hy[t] - q.y, hz[t] - q.z,
-                                          px, py, pz);
-                            }
-                        }
-                        rx[t - 1] += px; ry[t - 1] += py; rz[t - 1] += pz;
-                    }
-                    float2 *rw = slots + ((k & 1) * N * n_slots) * kPB + j;
-                    int i2 = i;
-                    for (int d = 0; d < n_pairs; ++d) {
-                        i2 = (i2 + 1 == N) ? 0 : i2 + 1;
-                        float2 ps = make_float2(0.0f, 0.0f);
-                        const float4 q = buf[i2 * kPB + j];
-                        const float dx = r.x - q.x, dy = r.y - q.y, dz = r.z - q.z;
-                        // beyond reach the penalty and its weight are below e^-30: 0,
-                        // as in the rollout; only a warp with a lane in reach evaluates
-                        const bool near = act && fmaf(dx, dx, dy * dy) < P.sp_far_h2 && fabsf(dz) < P.sp_far_v;
-                        if (__any_sync(0xffffffffu, near) && near) {
-                            ps = pair_penalty(P, dx, dy, dz);
-                            soft += ps.x;
-                            if (ps.y != 0.0f) pair_grad(P, sep_c * ps.y, dx, dy, dz, sx, sy, sz);
-                        }
-                        rw[(i2 * n_slots + d) * kPB] = ps;
-                    }
-                } else if (act) {
-                    for (int i2 = 0; i2 < N; ++i2) {
-                        if (i2 == i) continue;
-                        const float4 q = buf[i2 * kPB + j];
-                        const float dx = r.x - q.x, dy = r.y - q.y, dz = r.z - q.z;
-                        if (fmaf(dx, dx, dy * dy) >= P.sp_far_h2 || fabsf(dz) >= P.sp_far_v) continue;   // out of reach
-                        const float2 ps = pair_penalty(P, dx, dy, dz);
-                        soft += ps.x;
-                        if (ps.y != 0.0f) pair_grad(P, sep_c * ps.y, dx, dy, dz, sx, sy, sz);
-                    }
-                }
-                rx[t] = sx; ry[t] = sy; rz[t] = sz; rv[t] = sv; rc[t] = sc;
-            }
-            if (pair_once) {
-                // pairs of the interval's last step, received after one more barrier
-                tile_barrier(0, blockDim.x);
-                const int k = k1 - 1, t = k - k0;
-                const float2 *rr = slots + (((k & 1) * N + i) * n_slots) * kPB + j;
-                const float4 *pb = pos + (k % 3) * plane;
-                float px = 0.f, py = 0.f, pz = 0.f;
-                int o = i;
-                for (int d = 0; d < n_recv; ++d) {
-                    o = (o == 0) ? N - 1 : o - 1;
-                    const float2 ps = rr[d * kPB];
-                    soft += ps.x;
-                    if (ps.y != 0.0f) {
-                        const float4 q = pb[o * kPB + j];
-                        pair_grad(P, sep_c * ps.y, r.x - q.x, r.y - q.y, r.z - q.z, px, py, pz);
-                    }
-                }
-                rx[t] += px; ry[t] += py; rz[t] += pz;
-            }
-            // reverse sweep of the interval
-            for (int k = k1 - 1; k >= k0; --k) {
-                const int t = k - k0;
-                if (!((upd >> t) & 1u)) continue;
-                X += rx[t]; Y += ry[t]; Z += rz[t]; V += rv[t]; CH += rc[t];
-                const int sg = (k * P.S) / P.H;
-                if (sg != gseg) {
-                    if (gseg >= 0 && exists) {
-                        gout[3 * gseg] += gw;
-                        gout[3 * gseg + 1] += gh;
-                        gout[3 * gseg + 2] += ga;
-                    }
-                    gseg = sg;
-                    gw = gh = ga = 0.f;
-                }
-                step_adjoint(P, A, Wm + (size_t)k * P.P, hx[t], hy[t], hz[t], hv[t], hc[t],
-                             m0 - hF[t], __ldg(ul + 3 * sg), __ldg(ul + 3 * sg + 1),
-                             __ldg(ul + 3 * sg + 2), X, Y, Z, V, CH, FF, gw, gh, ga);
-            }
-        }
-        if (gseg >= 0 && exists) {
-            gout[3 * gseg] += gw;
-            gout[3 * gseg + 1] += gh;
-            gout[3 * gseg + 2] += ga;
-        }
-        if (exists)
-            cost_ms[((size_t)m * N + i) * (size_t)L + l] =
-                dead ? __int_as_float(0x7f800000) : fmaf(P.mu_sep, soft, c);
-    }
-}
-
-// One warp per particle: per-aircraft sample means (as the rollout's sample
-// mean: compensated, in sample order, +inf when any sample was infeasible),
-// their sum C_l, and the gradient summed over the sample ranges (zero when the
-// particle is infeasible).
-__global__ void __launch_bounds__(256) grad_reduce_kernel(const float *__restrict__ cost_ms,
-                                                          const float *__restrict__ gpart,
-                                                          long long L, int M, int N, int nS3,
-                                                          int nchunk, float *__restrict__ cost,
-                                                          float *__restrict__ grad,
-                                                          float *__restrict__ cbar)
-{
-    const long long l = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (l >= L) return;
-    float cb = 0.0f;
-    bool inf = false;
-    if (lane < N) {
+    constexpr int KC = 4;
+    __shared__ float means[256];
+    grid_begin();
+    const int N = P.N, H = P.H, B = N * TP, nS3 = P.S * 3;
+    const int t = threadIdx.x, i = t / TP, j = t % TP;
+    const int tile = blockIdx.x;
+    const long long l = l_begin + (long long)tile * TP + j;
+    // this aircraft's sample mean (as the rollout's: compensated, in sample order,
+    // +inf when any sample was infeasible), then the particle's sum C_l
+    float cb = __int_as_float(0x7f800000);
+    if (l < l_end) {
         Kahan s;
-        for (int m = 0; m < M; ++m) {
-            const float v = __ldg(cost_ms + ((size_t)m * N + lane) * (size_t)L + l);
+        bool inf = false;
+#pragma unroll 8
+        for (int m = 0; m < P.M; ++m) {
+            const float v = __ldg(cost_ms + ((size_t)m * N + i) * (size_t)L + l);
             if (isinf(v)) inf = true;
             else s.add(v);
         }
-        cb = inf ? __int_as_float(0x7f800000) : s.s / (float)M;
-        if (cbar) cbar[(size_t)lane * L + l] = cb;
+        if (!inf) cb = s.s / (float)P.M;
+        if (cbar) cbar[(size_t)i * L + l] = cb;
     }
-    const bool infeasible = __any_sync(0xffffffffu, inf);
-    double tot = lane < N && !inf ? (double)cb : 0.0;
+    means[t] = cb;
+    __syncthreads();
+    if (l >= l_end) return;
+    bool infeasible = false;
+    for (int q = 0; q < N; ++q) infeasible = infeasible || isinf(means[q * TP + j]);
+    if (i == 0) {
+        double tot = 0.0;
+        for (int q = 0; q < N; ++q) tot += (double)means[q * TP + j];
+        cost[l] = infeasible ? __int_as_float(0x7f800000) : (float)tot;
+    }
+    float *gout = grad + ((size_t)l * N + i) * (size_t)nS3;
+    for (int n = 0; n < nS3; ++n) gout[n] = 0.0f;
+    if (infeasible) return;
+    const AircraftC A = P.ac[i];
+    const float m0 = dyn->x0[i][5];
+    const float *ul = u + ((size_t)l * N + i) * (size_t)nS3;
+    const float4 *state = R.state + (size_t)tile * H * B + t;
+    // every sample's flight has ended (in a landing) before a step beyond a limit
+    const int k_stop = __float_as_int(R.fin[(size_t)tile * B + t].w);
+    if (k_stop == 0) return;
+    float gB = 0.0f, gC = 0.0f, FF = 0.0f;
+    for (int c = 0; c < n_ranges; ++c) {
+        const float4 q = G.sums[((size_t)c * n_tiles + tile) * B + t];
+        gB += q.x;
+        gC += q.y;
+        FF += q.z;
+    }
+    float Z = 0.f, V = 0.f, CH = 0.f, gw = 0.f, gh = 0.f, ga = 0.f;
+    int seg = (int)((long long)(k_stop - 1) * P.S / H);                 // the segment of step k
+    int k_seg = (int)(((long long)seg * H + P.S - 1) / P.S);            // and its first step
+    float4 post = state[(size_t)(k_stop - 1) * B];                      // the state after step k
+    for (int kt = k_stop - 1; kt >= 0; kt -= KC) {
+        // four steps: the states before them and the sums over the ranges, all these
+        // loads in flight together (one after the other they are the kernel's time)
+        float4 pre[KC], a[KC];
+        float lf[KC];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    if (lane == 0) cost[l] = infeasible ? __int_as_float(0x7f800000) : (float)tot;
-    const int nel = N * nS3;
-    const size_t stride = (size_t)L * nel;
-    for (int n = lane; n < nel; n += 32) {
-        float g = 0.0f;
-        if (!infeasible)
-            for (int c = 0; c < nchunk; ++c) g += __ldg(gpart + c * stride + (size_t)l * nel + n);
-        grad[(size_t)l * nel + n] = g;
+        for (int e = 0; e < KC; ++e) {
+            const int k = kt - e;
+            pre[e] = k > 0 ? state[(size_t)(k - 1) * B]
+                           : make_float4(dyn->x0[i][2], dyn->x0[i][3], 0.0f, dyn->x0[i][4]);
+            a[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+            lf[e] = 0.0f;
+        }
+#pragma unroll 2
+        for (int c = 0; c < n_ranges; ++c) {
+            const size_t o = ((size_t)c * n_tiles + tile) * H * B + t;
+#pragma unroll
+            for (int e = 0; e < KC; ++e) {
+                const float4 q = G.acc[o + (size_t)max(kt - e, 0) * B];
+                a[e].x += q.x;
+                a[e].y += q.y;
+                a[e].z += q.z;
+                a[e].w += q.w;
+            }
+        }
+        if (A.type == 0) {
+#pragma unroll 2
+            for (int c = 0; c < n_ranges; ++c) {
+                const size_t o = ((size_t)c * n_tiles + tile) * H * B + t;
+#pragma unroll
+                for (int e = 0; e < KC; ++e) lf[e] += G.land[o + (size_t)max(kt - e, 0) * B];
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < KC; ++e) {
+            const int k = kt - e;
+            if (k < 0) break;
+            if (k < k_seg) {
+                gout[3 * seg] = gw;
+                gout[3 * seg + 1] = gh;
+                gout[3 * seg + 2] = ga;
+                gw = gh = ga = 0.0f;
+                --seg;
+                k_seg = (int)(((long long)seg * H + P.S - 1) / P.S);
+            }
+            const StepCoef c = step_coef(P, A, pre[e].x, pre[e].y, pre[e].w, m0 - pre[e].z, __ldg(ul + 3 * seg),
+                                         __ldg(ul + 3 * seg + 1), __ldg(ul + 3 * seg + 2));
+            Z += a[e].z;
+            CH += a[e].w;
+            FF += lf[e];
+            if (A.type != 0) {
+                Z = fmaf(gB, sgnf(post.x - A.Z), Z);
+                V = fmaf(gC, sgnf(post.y - A.vD), V);
+            }
+            const float proj = fmaf(c.cc, a[e].x, c.sc * a[e].y);      // along-track adjoint
+            const float fe = FF * c.e;                                  // fuel adjoint times d F'/d T
+            gw += fmaf(P.dt, CH, fe * c.wT);
+            gh += P.dt * Z + c.hP * proj + fe * c.hT;
+            ga += fmaf(P.dt, V, fe * c.aT);
+            V += c.vP * proj + FF * c.vT;
+            CH += c.cP * fmaf(-c.sc, a[e].x, c.cc * a[e].y);
+            Z += fe * c.zT;
+            FF -= fe * c.mT;
+            post = pre[e];
+        }
     }
+    gout[3 * seg] = gw;
+    gout[3 * seg + 1] = gh;
+    gout[3 * seg + 2] = ga;
 }
+
+// bytes of the scratch of n particles (a multiple of 32), and its places in a buffer
+size_t grad_bytes(const ProblemC &P, size_t n, int n_ranges)
+{
+    const size_t steps = n * (size_t)P.N * (size_t)P.H;
+    return traj_slab_bytes(P, n) + steps * sizeof(float4) +
+           (size_t)n_ranges * (steps * (2 * sizeof(float4) + 2 * sizeof(float2) + sizeof(float)) +
+                               n * (size_t)P.N * ((size_t)n_chunks(P.H) * sizeof(unsigned) + sizeof(float4)));
+}
+
+GradScratch grad_places(const ProblemC &P, size_t n, int n_ranges, void *ws, TrajOut &R)
+{
+    const size_t ac = n * (size_t)P.N, steps = ac * (size_t)P.H;
+    GradScratch G;
+    R = traj_records(P, n, ws);
+    R.state = reinterpret_cast<float4 *>(static_cast<char *>(ws) + traj_slab_bytes(P, n));
+    G.acc = R.state + steps;
+    G.log.sep = G.acc + steps * n_ranges;
+    G.sums = G.log.sep + steps * n_ranges;
+    G.log.xy = reinterpret_cast<float2 *>(G.sums + ac * n_ranges);
+    G.log.polar = G.log.xy + steps * n_ranges;
+    G.land = reinterpret_cast<float *>(G.log.polar + steps * n_ranges);
+    G.log.near = reinterpret_cast<unsigned *>(G.land + steps * n_ranges);
+    return G;
+}
+
+// f(kernel) for the variant's instance of grad_samples_kernel at this aircraft count
+template <class F>
+auto with_samples_kernel(int N, int variant, F f)
+{
+    const int tp = traj_tile(N);
+    if (variant == 0) {
+        if (tp == 32) return f(grad_samples_kernel<3, 32>);
+        return tp == 16 ? f(grad_samples_kernel<3, 16>) : f(grad_samples_kernel<3, 8>);
+    }
+    if (tp == 32) return f(grad_samples_kernel<4, 32>);
+    return tp == 16 ? f(grad_samples_kernel<4, 16>) : f(grad_samples_kernel<4, 8>);
+}
+
+size_t samples_smem(int N) { return (size_t)wind_rollout_words(N, traj_tile(N), true, false) * sizeof(float); }
 
 }  // namespace
 
-// Launch-bound variants (block size cap, minimum resident blocks per SM); the
-// register budget per thread is 65536 / (cap * blocks).  The variant is chosen
-// by timing (host side) among those whose cap fits the block (32 N threads).
-struct GradVariant {
-    int max_threads, min_blocks;
-};
-constexpr GradVariant kGradVariants[] = {{256, 1}, {256, 2}, {256, 3}, {384, 1}, {384, 2},
-                                         {512, 1}, {768, 1}, {1024, 1}};
-constexpr int kNumGradVariants = sizeof(kGradVariants) / sizeof(kGradVariants[0]);
-
+// Launch-bound variants of grad_samples_kernel: minimum resident blocks of 256
+// threads (80 and 64 registers a thread), chosen by timing.
 int rollout_grad_variants(int N, int *out)
 {
-    int n = 0;
-    for (int v = 0; v < kNumGradVariants; ++v)
-        if (kGradVariants[v].max_threads >= N * kPB) out[n++] = v;
-    return n;
-}
-
-#define TMA_GRAD_VARIANT_SWITCH(V, CALL)                              \
-    switch (V) {                                                      \
-    case 0: CALL(256, 1); break;                                      \
-    case 1: CALL(256, 2); break;                                      \
-    case 2: CALL(256, 3); break;                                      \
-    case 3: CALL(384, 1); break;                                      \
-    case 4: CALL(384, 2); break;                                      \
-    case 5: CALL(512, 1); break;                                      \
-    case 6: CALL(768, 1); break;                                      \
-    default: CALL(1024, 1); break;                                    \
-    }
-
-static int valid_variant(int N, int variant)
-{
-    if (variant >= 0 && variant < kNumGradVariants && kGradVariants[variant].max_threads >= N * kPB)
-        return variant;
-    int cand[kNumGradVariants];
-    rollout_grad_variants(N, cand);
-    return cand[0];
+    (void)N;
+    out[0] = 0;
+    out[1] = 1;
+    return 2;
 }
 
 cudaError_t rollout_grad_occupancy(int N, int variant, int *blocks_per_sm)
 {
-    const int block = N * kPB;
-    const size_t smem = (size_t)2 * 3 * N * kPB * sizeof(float);
-#define TMA_OCC(T, B)                                                                            \
-    do {                                                                                         \
-        if (smem > 48 * 1024)                                                                    \
-            cudaFuncSetAttribute(rollout_grad_kernel<T, B>,                                      \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, rollout_grad_kernel<T, B>, \
-                                                             block, smem);                       \
-    } while (0)
-    TMA_GRAD_VARIANT_SWITCH(valid_variant(N, variant), TMA_OCC)
-#undef TMA_OCC
-    return cudaSuccess;
+    return with_samples_kernel(N, variant, [&](auto kernel) {
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, N * traj_tile(N), samples_smem(N));
+    });
 }
 
-cudaError_t launch_rollout_grad(const ProblemC &P, const DynState *dyn, const float *u,
-                                const float *W, int64_t L, int J, int nchunk, float *cost_ms,
-                                float *gpart, float *cost, float *grad, float *cbar,
-                                cudaStream_t st, int variant)
+int rollout_grad_tile(int N) { return traj_tile(N); }
+
+size_t rollout_grad_workspace(const ProblemC &P, int64_t L, int n_ranges, size_t most)
+{
+    const size_t per32 = grad_bytes(P, 32, n_ranges);
+    const size_t want = ((size_t)L + 31) / 32, fit = most / per32;
+    return (want < fit ? want : (fit > 0 ? fit : 1)) * per32;
+}
+
+cudaError_t launch_rollout_grad(const ProblemC &P, const DynState *dyn, const float *u, const float *W, int64_t L,
+                                int J, int n_ranges, float *cost_ms, void *ws, size_t ws_bytes, float *cost, float *grad,
+                                float *cbar, cudaStream_t st, int variant)
 {
     if (L <= 0) return cudaSuccess;
-    const long long nLb = (L + kPB - 1) / kPB;
-    const int m_per_block = (P.M + nchunk - 1) / nchunk;
-    nchunk = (P.M + m_per_block - 1) / m_per_block;
-    const unsigned grid = (unsigned)(nLb * nchunk);
-    const int block = P.N * kPB;
-    const size_t smem = (size_t)grad_smem_words(P.N) * sizeof(float);
+    const int m_per_block = (P.M + n_ranges - 1) / n_ranges;
+    n_ranges = (P.M + m_per_block - 1) / m_per_block;
+    const size_t slab = ws_bytes / grad_bytes(P, 32, n_ranges) * 32, all = ((size_t)L + 31) / 32 * 32;
+    if (!ws || slab == 0) return cudaErrorInvalidValue;
+    const size_t n = slab < all ? slab : all;
+    TrajOut R;
+    const GradScratch G = grad_places(P, n, n_ranges, ws, R);
     const float4 *W4 = reinterpret_cast<const float4 *>(W);
-#define TMA_LAUNCH(T, B)                                                                   \
-    do {                                                                                   \
-        if (smem > 48 * 1024)                                                              \
-            cudaFuncSetAttribute(rollout_grad_kernel<T, B>,                                \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);  \
-        rollout_grad_kernel<T, B><<<grid, block, smem, st>>>(P, dyn, u, W4, L, (int)nLb,   \
-                                                             m_per_block, J, cost_ms, gpart); \
-    } while (0)
-    TMA_GRAD_VARIANT_SWITCH(valid_variant(P.N, variant), TMA_LAUNCH)
-#undef TMA_LAUNCH
-    count_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !cost) return e;
-    grad_reduce_kernel<<<(unsigned)((L * 32 + 255) / 256), 256, 0, st>>>(
-        cost_ms, gpart, L, P.M, P.N, P.S * 3, nchunk, cost, grad, cbar);
-    count_launch();
-    return cudaGetLastError();
+    const int tp = traj_tile(P.N), block = P.N * tp;
+    const size_t smem = samples_smem(P.N);
+    const auto slab_end = [&](int64_t l0) { return l0 + (int64_t)n < L ? l0 + (int64_t)n : L; };
+    for (int64_t l0 = 0; l0 < L; l0 += (int64_t)n) {
+        const long long l1 = slab_end(l0);
+        const int n_tiles = (int)((l1 - l0 + tp - 1) / tp);
+        launch_trajectories(P, dyn, u, l0, l1, R, true, st, true);
+        with_samples_kernel(P.N, variant, [&](auto kernel) {
+            launch_dependent(kernel, (unsigned)n_tiles * (unsigned)n_ranges, block, smem, st, P, dyn, W4, R, G, L, l0, l1,
+                             n_tiles, m_per_block, J, cost_ms);
+            return 0;
+        });
+        count_launch();
+        if (cost) {
+#define TMA_CONTROLS(TP)                                                                                              \
+    launch_dependent(grad_controls_kernel<TP>, n_tiles, block, 0, st, P, dyn, u, R, G, l0, l1, n_tiles, n_ranges,     \
+                     cost_ms, L, cost, grad, cbar)
+            if (tp == 32) TMA_CONTROLS(32);
+            else if (tp == 16) TMA_CONTROLS(16);
+            else TMA_CONTROLS(8);
+#undef TMA_CONTROLS
+            count_launch();
+        }
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace tma

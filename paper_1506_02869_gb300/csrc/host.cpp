@@ -358,7 +358,7 @@ static void free_all(tma_solver *s)
                     s->d_cost_ms_soft, s->d_cbar, s->d_cbar_soft, s->d_wtilde, s->d_anc,
                     s->d_popdense, s->d_work, s->d_best, s->d_best_sum, s->d_ninf, s->d_flags, s->d_err,
                     s->d_live, s->d_best_u, s->d_probs1, s->d_scen1, s->d_seg_scen1,
-                    s->d_gcost_ms, s->d_gpart, s->d_eps, s->d_nacc, s->d_acc_hist,
+                    s->d_gcost_ms, s->d_gwork, s->d_eps, s->d_nacc, s->d_acc_hist,
                     s->d_eps_hist, s->d_u_prop, s->d_grad0, s->d_grad1, s->d_cbar0, s->d_cbar1,
                     s->d_cost0, s->d_cost1, s->d_inbox, s->d_traj};
     for (void *p : ptrs)
@@ -979,11 +979,15 @@ tma_status tma_init_controls(tma_solver *s, float *d_u, int64_t L, tma_stream_t 
 // waves of the device, at most one range per sample.
 static int grad_chunks(tma_solver *s, int64_t L, int variant, int M)
 {
-    int sms = 0, per_sm = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
-    if (rollout_grad_occupancy(s->prob.N, variant, &per_sm) != cudaSuccess || per_sm < 1) per_sm = 1;
-    const long long tiles = (L + kTileParticles - 1) / kTileParticles;
-    const long long want = 2LL * std::max(sms, 1) * per_sm;
+    if (s->grad_slots[variant] == 0) {           // resident blocks of the device, asked once
+        int sms = 0, per_sm = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
+        if (rollout_grad_occupancy(s->prob.N, variant, &per_sm) != cudaSuccess || per_sm < 1) per_sm = 1;
+        s->grad_slots[variant] = std::max(sms, 1) * per_sm;
+    }
+    const int tp = rollout_grad_tile(s->prob.N);
+    const long long tiles = (L + tp - 1) / tp;
+    const long long want = 2LL * s->grad_slots[variant];
     long long c = (want + tiles - 1) / std::max(tiles, 1LL);
     return (int)std::max(1LL, std::min<long long>(c, M));
 }
@@ -995,15 +999,27 @@ static tma_status ensure_grad_scratch(tma_solver *s, int64_t L, int nchunk)
         cudaError_t e = alloc(&s->d_gcost_ms, (size_t)p.M * p.N * p.L * sizeof(float));
         if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TMA_ERR_OOM : record_cuda_error(e);
     }
-    const size_t need = (size_t)nchunk * L * p.N * p.S * 3;
-    if (need > s->gpart_elems) {
-        if (s->d_gpart) cudaFree(s->d_gpart);
-        s->d_gpart = nullptr;
-        s->gpart_elems = 0;
-        cudaError_t e = alloc(&s->d_gpart, need * sizeof(float));
-        if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TMA_ERR_OOM : record_cuda_error(e);
-        s->gpart_elems = need;
+    // 2 GB at most (larger particle counts run in slabs); on a nearly full device
+    // half as much again and again, down to the smallest slab
+    const ProblemC &P = s->P;
+    size_t want = rollout_grad_workspace(P, L, nchunk, (size_t)2 << 30);
+    const size_t asked = want, least = rollout_grad_workspace(P, 1, nchunk, 0);
+    if (want <= s->gwork_asked) return TMA_OK;
+    s->gwork_asked = 0;
+    if (s->d_gwork) cudaFree(s->d_gwork);
+    s->d_gwork = nullptr;
+    s->gwork_bytes = 0;
+    for (;;) {
+        const cudaError_t e = cudaMalloc(&s->d_gwork, want);
+        if (e == cudaSuccess) break;
+        s->d_gwork = nullptr;
+        if (e != cudaErrorMemoryAllocation) return record_cuda_error(e);
+        cudaGetLastError();
+        if (want <= least) return TMA_ERR_OOM;
+        want = std::max(least, want / 2);
     }
+    s->gwork_bytes = want;
+    s->gwork_asked = asked;
     return TMA_OK;
 }
 
@@ -1055,12 +1071,12 @@ static tma_status autotune_grad(tma_solver *s)
     for (int c = 0; c < nc && e == cudaSuccess; ++c) {
         const int nch = grad_chunks(s, Lp, cand[c], s->prob.M);
         // one untimed launch, then two timed
-        e = launch_rollout_grad(s->P, s->d_dyn, d_u, s->d_W, Lp, 0, nch, s->d_gcost_ms, s->d_gpart,
-                                nullptr, nullptr, nullptr, st, cand[c]);
+        e = launch_rollout_grad(s->P, s->d_dyn, d_u, s->d_W, Lp, 0, nch, s->d_gcost_ms, s->d_gwork,
+                                s->gwork_bytes, nullptr, nullptr, nullptr, st, cand[c]);
         if (e == cudaSuccess) e = cudaEventRecord(e0, st);
         for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep)
             e = launch_rollout_grad(s->P, s->d_dyn, d_u, s->d_W, Lp, 0, nch, s->d_gcost_ms,
-                                    s->d_gpart, nullptr, nullptr, nullptr, st, cand[c]);
+                                    s->d_gwork, s->gwork_bytes, nullptr, nullptr, nullptr, st, cand[c]);
         if (e == cudaSuccess) e = cudaEventRecord(e1, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.0f;
@@ -1100,7 +1116,7 @@ static tma_status grad_into(tma_solver *s, const float *d_u, int64_t L, int32_t 
     if (r != TMA_OK) return r;
     StageTimer t(s, 8, st);
     TMA_CUDA(launch_rollout_grad(Pj, s->d_dyn, d_u, s->d_W, L, J, nchunk, s->d_gcost_ms,
-                                 s->d_gpart, cost, grad, cbar, st, s->grad_variant));
+                                 s->d_gwork, s->gwork_bytes, cost, grad, cbar, st, s->grad_variant));
     return TMA_OK;
 }
 

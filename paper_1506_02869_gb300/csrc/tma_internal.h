@@ -196,16 +196,18 @@ cudaError_t launch_gather_best(const float *u, const int64_t *best, int nctl_per
                                float *best_u, cudaStream_t st, const unsigned int *flags = nullptr,
                                const int *ninf = nullptr, unsigned int *err = nullptr);
 
-// gradient of the soft cost (adjoint.cu): per-sample costs cost_ms[M][N][L],
-// partial gradients gpart[nchunk][L][N][S][3] over nchunk ranges of samples
-// (cost == nullptr: the main kernel only, for timing); variant indexes the
-// launch-bound table (rollout_grad_variants lists those valid for N)
-cudaError_t launch_rollout_grad(const ProblemC &P, const DynState *dyn, const float *u,
-                                const float *W, int64_t L, int J, int nchunk, float *cost_ms,
-                                float *gpart, float *cost, float *grad, float *cbar,
-                                cudaStream_t st, int variant);
+// gradient of the soft cost (adjoint.cu): per-sample costs cost_ms[M][N][L]; ws: its
+// scratch, of which rollout_grad_workspace says how much L particles in n_ranges
+// ranges of samples want (at most `most`, but at least 32 particles' share: more run in
+// slabs); (cost == nullptr: the kernels over the samples only, for timing); variant
+// indexes the launch-bound table
+cudaError_t launch_rollout_grad(const ProblemC &P, const DynState *dyn, const float *u, const float *W, int64_t L,
+                                int J, int n_ranges, float *cost_ms, void *ws, size_t ws_bytes, float *cost, float *grad,
+                                float *cbar, cudaStream_t st, int variant);
+size_t rollout_grad_workspace(const ProblemC &P, int64_t L, int n_ranges, size_t most);
 cudaError_t rollout_grad_occupancy(int N, int variant, int *blocks_per_sm);
 int rollout_grad_variants(int N, int *out);
+int rollout_grad_tile(int N);      // particles per block
 
 // Metropolis-Hastings moves (mala.cu)
 cudaError_t launch_mh_propose(const MhParams &h, const DynState *dyn, const float *u,
@@ -310,8 +312,9 @@ struct tma_solver {
     int *d_seg_scen1 = nullptr;
     // gradient scratch (allocated on first use)
     float *d_gcost_ms = nullptr;        // [M][N][L]
-    float *d_gpart = nullptr;           // [nchunk][L][N][S][3]
-    size_t gpart_elems = 0;
+    void *d_gwork = nullptr;            // the kernels' scratch (rollout_grad_workspace)
+    size_t gwork_bytes = 0, gwork_asked = 0;
+    int grad_slots[8] = {0};            // resident blocks of each variant on the device (0: not asked yet)
     int grad_variant = -1;              // autotuned launch variant of the gradient kernel
     int n_grad_tuned = 0;
     int grad_tuned_variant[8] = {0};
