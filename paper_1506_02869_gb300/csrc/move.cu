@@ -6,6 +6,7 @@
 // u[anc[i][l]][i] is gathered with 16-byte loads (S*3 = 12 floats = 3 x float4
 // when S = 4); the Gaussian noise comes from random stream 1.
 #include "device_common.cuh"
+#include "launch.cuh"
 #include "tma_internal.h"
 
 namespace tma {
@@ -32,6 +33,7 @@ __global__ void __launch_bounds__(256) move_kernel(const MoveC C, const DynState
                                                    unsigned int *__restrict__ err)
 {
     // L children from Lin parents
+    grid_begin();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L * C.N) return;
     const long long l = t / C.N;
@@ -127,9 +129,9 @@ cudaError_t launch_move(const ProblemC &P, const DynState *dyn, const float ctrl
     const MoveC C = make_move(P, ctrl_lo, ctrl_hi, sigma);
     const long long n = (long long)L * P.N;
     const unsigned grid = (unsigned)((n + 255) / 256);
-    if (C.nc == 12) move_kernel<true, 12><<<grid, 256, 0, st>>>(C, dyn, u, anc, L, Lin, J, u_out, err);
-    else if (C.nc % 4 == 0) move_kernel<true><<<grid, 256, 0, st>>>(C, dyn, u, anc, L, Lin, J, u_out, err);
-    else move_kernel<false><<<grid, 256, 0, st>>>(C, dyn, u, anc, L, Lin, J, u_out, err);
+    if (C.nc == 12) launch_dependent(move_kernel<true, 12>, grid, 256, 0, st, C, dyn, u, anc, L, Lin, J, u_out, err);
+    else if (C.nc % 4 == 0) launch_dependent(move_kernel<true>, grid, 256, 0, st, C, dyn, u, anc, L, Lin, J, u_out, err);
+    else launch_dependent(move_kernel<false>, grid, 256, 0, st, C, dyn, u, anc, L, Lin, J, u_out, err);
     count_launch();
     return cudaGetLastError();
 }

@@ -36,6 +36,7 @@
 
 #include "device_common.cuh"
 #include "exp_table.h"
+#include "launch.cuh"
 #include "tma_internal.h"
 
 namespace tma {
@@ -99,6 +100,7 @@ __global__ void __launch_bounds__(kThreads) lse_chunk_min(const float *__restric
                                                           int nchunk, float *__restrict__ cmin)
 {
     __shared__ float sh[32];
+    grid_begin();
     const int s = blockIdx.y, c = blockIdx.x;
     const float *row = cbar + (size_t)s * L;
     const long long base = (long long)c * kChunk;
@@ -212,7 +214,8 @@ __global__ void __launch_bounds__(kThreads) lse_exp(const float *__restrict__ cb
     __shared__ unsigned long long shq[32];
     __shared__ unsigned long long tab[256];
     const int s = blockIdx.y, c = blockIdx.x;
-    for (int j = threadIdx.x; j < 256; j += kThreads) tab[j] = kExp2Frac63[j];
+    for (int j = threadIdx.x; j < 256; j += kThreads) tab[j] = kExp2Frac63[j];      // constants of the library
+    grid_begin();
     float mn = __int_as_float(0x7f800000);
     for (int j = threadIdx.x; j < nchunk; j += kThreads) mn = fminf(mn, cmin[(size_t)s * nchunk + j]);
     mn = block_reduce(mn, MinOp(), shf, __int_as_float(0x7f800000));   // its barriers also cover tab
@@ -260,6 +263,7 @@ __global__ void lse_finish(const float *__restrict__ cmin, const double *__restr
                            int nchunk, double kappa, double *__restrict__ lmax,
                            double *__restrict__ wsum)
 {
+    grid_begin();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nseg) return;
     float mn = __int_as_float(0x7f800000);
@@ -277,6 +281,7 @@ __global__ void __launch_bounds__(kThreads) res_chunk_sum(const double *__restri
                                                           unsigned long long *__restrict__ cq)
 {
     __shared__ unsigned long long sh[32];
+    grid_begin();
     const int s = blockIdx.y, c = blockIdx.x;
     const double *row = wtilde + (size_t)s * L;
     const long long base = (long long)c * kChunk;
@@ -427,6 +432,7 @@ __global__ void __launch_bounds__(kThreads) res_expand(const double *__restrict_
     __shared__ unsigned long long seg_before, seg_total;
     __shared__ Thresholds Tsh;
     __shared__ ChunkBase Bsh;
+    grid_begin();
     const int s = blockIdx.y, c = blockIdx.x;
     const long long base = (long long)c * kChunk;
     const int len = (int)min((long long)kChunk, L - base);
@@ -660,11 +666,11 @@ cudaError_t launch_lse(const float *cbar, int nseg, int64_t L, double kappa, dou
     double *csum = reinterpret_cast<double *>(
         (reinterpret_cast<uintptr_t>(cmin + n) + 15) & ~uintptr_t(15));
     dim3 grid(nc, nseg);
-    lse_chunk_min<<<grid, kThreads, 0, st>>>(cbar, L, nc, cmin);
-    lse_exp<<<grid, kThreads, 0, st>>>(cbar, L, nc, kappa, cmin, wtilde, (lmax || wsum) ? csum : nullptr, cq);
+    launch_dependent(lse_chunk_min, grid, kThreads, 0, st, cbar, L, nc, cmin);
+    launch_dependent(lse_exp, grid, kThreads, 0, st, cbar, L, nc, kappa, cmin, wtilde, (lmax || wsum) ? csum : nullptr, cq);
     count_launch(2);
     if (lmax || wsum) {
-        lse_finish<<<(nseg + 127) / 128, 128, 0, st>>>(cmin, csum, nseg, nc, kappa, lmax, wsum);
+        launch_dependent(lse_finish, (nseg + 127) / 128, 128, 0, st, cmin, csum, nseg, nc, kappa, lmax, wsum);
         count_launch();
     }
     return cudaGetLastError();
@@ -756,11 +762,11 @@ cudaError_t launch_resample(const double *wtilde, int nseg, int64_t L, int64_t L
     unsigned long long *cq = resample_partials(work);
     dim3 grid(nc, nseg);
     if (!sums_ready) {
-        res_chunk_sum<<<grid, kThreads, 0, st>>>(wtilde, L, nc, cq);
+        launch_dependent(res_chunk_sum, grid, kThreads, 0, st, wtilde, L, nc, cq);
         count_launch();
     }
-    res_expand<<<grid, kThreads, 0, st>>>(wtilde, L, Lout, nc, cq, key0, key1, J, d_mpc, mpc_host,
-                                          anc, d_flags, seg_keys, dyns);
+    launch_dependent(res_expand, grid, kThreads, 0, st, wtilde, L, Lout, nc, cq, key0, key1, J, d_mpc, mpc_host, anc,
+                     d_flags, seg_keys, dyns);
     count_launch();
     return cudaGetLastError();
 }

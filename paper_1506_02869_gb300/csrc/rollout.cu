@@ -11,6 +11,7 @@
 // positions of the same particle from shared memory (double-buffered by step,
 // one barrier per step).  Blocks are ordered with the wind sample slowest, so
 // the blocks resident at one time read the same wind field and share it in L2.
+#include "launch.cuh"
 #include "rollout_tile.cuh"
 
 namespace tma {
@@ -34,6 +35,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) rollout_kernel(const 
                                                        unsigned long long *__restrict__ live)
 {
     extern __shared__ float spos[];
+    grid_begin();
     const int m = blockIdx.x / nLb;            // wind sample: block-uniform
     const long long l0 = (long long)(blockIdx.x - m * nLb) * TP;
     const int i = threadIdx.x / TP, j = threadIdx.x % TP;
@@ -48,6 +50,7 @@ __global__ void __launch_bounds__(256) sample_mean_kernel(const float *__restric
                                                           long long L, int M, int N,
                                                           float *__restrict__ cbar)
 {
+    grid_begin();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L * N) return;
     Kahan s;
@@ -139,14 +142,14 @@ static void launch_small_tile(const ProblemC &P, const DynState *dyn, const floa
         if (smem > 48 * 1024)
             cudaFuncSetAttribute(rollout_kernel<T, B, false, false, true, TP>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        rollout_kernel<T, B, false, false, true, TP><<<grid, block, smem, st>>>(P, dyn, u, W4, L, (int)nLb, J,
-                                                                              cost_ms, cost_ms_soft, live);
+        launch_dependent(rollout_kernel<T, B, false, false, true, TP>, grid, block, smem, st, P, dyn, u, W4, L,
+                         (int)nLb, J, cost_ms, cost_ms_soft, live);
     } else {
         if (smem > 48 * 1024)
             cudaFuncSetAttribute(rollout_kernel<T, B, false, false, false, TP>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        rollout_kernel<T, B, false, false, false, TP><<<grid, block, smem, st>>>(P, dyn, u, W4, L, (int)nLb, J,
-                                                                               cost_ms, cost_ms_soft, live);
+        launch_dependent(rollout_kernel<T, B, false, false, false, TP>, grid, block, smem, st, P, dyn, u, W4, L,
+                         (int)nLb, J, cost_ms, cost_ms_soft, live);
     }
 }
 
@@ -200,8 +203,8 @@ cudaError_t launch_rollout(const ProblemC &P, const DynState *dyn, const float *
         if (smem > 48 * 1024)                                                                    \
             cudaFuncSetAttribute(rollout_kernel<T, B, O, R, F>,                                  \
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
-        rollout_kernel<T, B, O, R, F><<<grid, block, smem, st>>>(P, dyn, u, W4, L, (int)nLb, J,  \
-                                                                 cost_ms, cost_ms_soft, live);   \
+        launch_dependent(rollout_kernel<T, B, O, R, F>, grid, block, smem, st, P, dyn, u, W4, L, \
+                         (int)nLb, J, cost_ms, cost_ms_soft, live);                              \
     } while (0)
 #define TMA_ROLLOUT_K(T, B, O, R)                                                                \
     do {                                                                                         \
@@ -240,7 +243,7 @@ cudaError_t launch_sample_mean(const float *cost_ms, int64_t L, int M, int N, fl
 {
     if (L <= 0) return cudaSuccess;
     const long long n = (long long)L * N;
-    sample_mean_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(cost_ms, L, M, N, cbar);
+    launch_dependent(sample_mean_kernel, (unsigned)((n + 255) / 256), 256, 0, st, cost_ms, L, M, N, cbar);
     count_launch();
     return cudaGetLastError();
 }

@@ -4,6 +4,7 @@
 // one block over the candidates.  Sums run over aircraft in index order in
 // FP64, so the decision is exact and independent of the launch shape.
 #include "device_common.cuh"
+#include "launch.cuh"
 #include "tma_internal.h"
 
 namespace tma {
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(256) select_partial(const float *__restrict__ 
 {
     __shared__ int wn[8];
     __shared__ float wh[8];
+    grid_begin();
     Cand best{1 << 30, 0.0, 1ll << 62};
     int bn = 1 << 30;                                  // least infeasible count of the block so far,
     float bh = __int_as_float(0x7f800000);             // least upper end among those
@@ -146,6 +148,7 @@ __global__ void __launch_bounds__(256) select_final(const Cand *__restrict__ par
                                                     double *__restrict__ out_sum,
                                                     int *__restrict__ out_ninf)
 {
+    grid_begin();
     Cand best{1 << 30, 0.0, 1ll << 62};
     for (int j = threadIdx.x; j < nparts; j += blockDim.x)
         if (better(part[j], best)) best = part[j];
@@ -164,6 +167,7 @@ __global__ void gather_best_kernel(const float *__restrict__ u, const long long 
                                    int n, float *__restrict__ out, const unsigned int *flags,
                                    const int *ninf, unsigned int *err)
 {
+    grid_begin();
     const long long b = *best;
     for (int j = threadIdx.x; j < n; j += blockDim.x) out[j] = u[(size_t)b * n + j];
     if (err && threadIdx.x == 0) *err |= (*flags & 1u) | (*ninf > 0 ? 2u : 0u);
@@ -186,8 +190,8 @@ cudaError_t launch_select(const float *cbar, int N, int64_t L, int64_t *best, do
     auto *part = reinterpret_cast<Cand *>((reinterpret_cast<uintptr_t>(work) + 15) & ~uintptr_t(15));
     const long long need = (L + 255) / 256;
     const int nb = (int)(need < kSelBlocks ? need : kSelBlocks);
-    select_partial<<<nb, 256, 0, st>>>(cbar, N, L, part);
-    select_final<<<1, 256, 0, st>>>(part, nb, reinterpret_cast<long long *>(best), best_sum, ninf);
+    launch_dependent(select_partial, nb, 256, 0, st, cbar, N, L, part);
+    launch_dependent(select_final, 1, 256, 0, st, part, nb, reinterpret_cast<long long *>(best), best_sum, ninf);
     count_launch(2);
     return cudaGetLastError();
 }
@@ -196,8 +200,8 @@ cudaError_t launch_gather_best(const float *u, const int64_t *best, int n, float
                                cudaStream_t st, const unsigned int *flags, const int *ninf,
                                unsigned int *err)
 {
-    gather_best_kernel<<<1, 256, 0, st>>>(u, reinterpret_cast<const long long *>(best), n, best_u,
-                                          flags, ninf, err);
+    launch_dependent(gather_best_kernel, 1, 256, 0, st, u, reinterpret_cast<const long long *>(best), n, best_u, flags,
+                     ninf, err);
     count_launch();
     return cudaGetLastError();
 }
