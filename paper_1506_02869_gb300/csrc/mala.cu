@@ -11,6 +11,7 @@
 // are rejected; the accept test uses one uniform of stream 6 and is taken in
 // FP64.  One warp per particle: lanes run over the N * S * 3 controls.
 #include "device_common.cuh"
+#include "launch.cuh"
 #include "tma_internal.h"
 
 namespace tma {
@@ -37,6 +38,7 @@ __global__ void __launch_bounds__(256) mh_propose_kernel(MhParams h, const DynSt
                                                          float *__restrict__ u_prop,
                                                          uint8_t *__restrict__ inbox)
 {
+    grid_begin();
     const long long l = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (l >= L) return;
@@ -76,6 +78,7 @@ __global__ void __launch_bounds__(256) mh_accept_kernel(
     float *__restrict__ cbar_out, uint8_t *__restrict__ accepted,
     unsigned int *__restrict__ n_accept)
 {
+    grid_begin();
     const long long l = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (l >= L) return;
@@ -142,6 +145,7 @@ __global__ void __launch_bounds__(256) mh_accept_kernel(
 __global__ void mh_adapt_kernel(double *eps, unsigned int *n_accept, unsigned int *history,
                                 double *eps_history, int J, long long L)
 {
+    grid_begin();
     const double rate = (double)*n_accept / (double)L;
     if (history) history[J] = *n_accept;
     if (eps_history) eps_history[J] = *eps;
@@ -157,8 +161,7 @@ cudaError_t launch_mh_propose(const MhParams &h, const DynState *dyn, const floa
                               float *u_prop, uint8_t *inbox, cudaStream_t st)
 {
     if (L <= 0) return cudaSuccess;
-    mh_propose_kernel<<<(unsigned)((L * 32 + 255) / 256), 256, 0, st>>>(h, dyn, u, grad, L, J, kappa,
-                                                                        d_eps, u_prop, inbox);
+    launch_dependent(mh_propose_kernel, (unsigned)((L * 32 + 255) / 256), 256, 0, st, h, dyn, u, grad, L, J, kappa, d_eps, u_prop, inbox);
     count_launch();
     return cudaGetLastError();
 }
@@ -170,9 +173,7 @@ cudaError_t launch_mh_accept(const MhParams &h, const DynState *dyn, const float
                              unsigned int *n_accept, cudaStream_t st)
 {
     if (L <= 0) return cudaSuccess;
-    mh_accept_kernel<<<(unsigned)((L * 32 + 255) / 256), 256, 0, st>>>(
-        h, dyn, u, up, cbar, cbarp, g, gp, inbox, L, J, kappa, d_eps, u_out, cbar_out, accepted,
-        n_accept);
+    launch_dependent(mh_accept_kernel, (unsigned)((L * 32 + 255) / 256), 256, 0, st, h, dyn, u, up, cbar, cbarp, g, gp, inbox, L, J, kappa, d_eps, u_out, cbar_out, accepted, n_accept);
     count_launch();
     return cudaGetLastError();
 }
@@ -180,7 +181,7 @@ cudaError_t launch_mh_accept(const MhParams &h, const DynState *dyn, const float
 cudaError_t launch_mh_adapt(double *eps, unsigned int *n_accept, unsigned int *history,
                             double *eps_history, int J, int64_t L, cudaStream_t st)
 {
-    mh_adapt_kernel<<<1, 1, 0, st>>>(eps, n_accept, history, eps_history, J, L);
+    launch_dependent(mh_adapt_kernel, 1, 1, 0, st, eps, n_accept, history, eps_history, J, L);
     count_launch();
     return cudaGetLastError();
 }

@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(256) move_kernel(const MoveC C, const DynState
 __global__ void __launch_bounds__(256) init_kernel(const MoveC C, const DynState *__restrict__ dyn,
                                                    long long L, float *__restrict__ u)
 {
+    grid_begin();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L * C.N) return;
     const long long l = t / C.N;
@@ -142,7 +143,7 @@ cudaError_t launch_init_controls(const ProblemC &P, const DynState *dyn, const f
     if (L <= 0) return cudaSuccess;
     const MoveC C = make_move(P, ctrl_lo, ctrl_hi, nullptr);
     const long long n = (long long)L * P.N;
-    init_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(C, dyn, L, u);
+    launch_dependent(init_kernel, (unsigned)((n + 255) / 256), 256, 0, st, C, dyn, L, u);
     count_launch();
     return cudaGetLastError();
 }

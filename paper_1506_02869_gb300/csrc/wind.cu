@@ -12,6 +12,7 @@
 // level up, so that the trilinear interpolation needs four aligned 16-byte
 // loads and no subtraction in the vertical direction; the plain values too
 // when the caller wants them.
+#include "launch.cuh"
 #include "wind_normals.cuh"
 
 namespace tma {
@@ -22,6 +23,7 @@ template <int LANES>
 __global__ void __launch_bounds__(128) wind_normals_ar_kernel(const WindC w, const DynState *__restrict__ dyn,
                                                               float *__restrict__ Btmp)
 {
+    grid_begin();
     const long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
     const int iz = threadIdx.x % LANES;
     const bool on = t < (long long)w.M * w.nxy && iz < w.nz;
@@ -74,6 +76,7 @@ __global__ void __launch_bounds__(T *T / 64, 6)
     constexpr int kThreads = T * T / 64, kPad = T + 2;   // rows an odd number of 8-byte words apart: no bank conflicts along rows
     constexpr int kRing = kStages * kKStep * 2 * T, kOut = 64 * kPad;
     __shared__ __align__(16) float sh[kRing > kOut ? kRing : kOut];
+    grid_begin();
     const int t = threadIdx.x;
     const int tx = t % (T / 8), ty = t / (T / 8);
     const int rt = n_rtiles - 1 - (int)(blockIdx.x / n_ctiles);
@@ -180,10 +183,10 @@ cudaError_t launch_wind_normals_ar(const WindC &w, const DynState *dyn, float *B
     const int lanes = wind_column_lanes(w.nz);
     const unsigned grid = (unsigned)(((long long)w.M * w.nxy * lanes + 127) / 128);
     switch (lanes) {
-    case 2: wind_normals_ar_kernel<2><<<grid, 128, 0, st>>>(w, dyn, Btmp); break;
-    case 4: wind_normals_ar_kernel<4><<<grid, 128, 0, st>>>(w, dyn, Btmp); break;
-    case 8: wind_normals_ar_kernel<8><<<grid, 128, 0, st>>>(w, dyn, Btmp); break;
-    default: wind_normals_ar_kernel<16><<<grid, 128, 0, st>>>(w, dyn, Btmp); break;
+    case 2: launch_dependent(wind_normals_ar_kernel<2>, grid, 128, 0, st, w, dyn, Btmp); break;
+    case 4: launch_dependent(wind_normals_ar_kernel<4>, grid, 128, 0, st, w, dyn, Btmp); break;
+    case 8: launch_dependent(wind_normals_ar_kernel<8>, grid, 128, 0, st, w, dyn, Btmp); break;
+    default: launch_dependent(wind_normals_ar_kernel<16>, grid, 128, 0, st, w, dyn, Btmp); break;
     }
     count_launch();
     return cudaGetLastError();
@@ -195,8 +198,8 @@ cudaError_t launch_wind_gemm(const WindC &w, const float *Lxy_t, int lda, const 
     constexpr int T = 64;
     const int cols = wind_tile_cols(T, w.nz);
     const int ct = (w.ncol + cols - 1) / cols, rt = (w.nxy + T - 1) / T;
-    wind_gemm_kernel<T><<<ct * rt, T * T / 64, 0, st>>>(w, Lxy_t, lda, Btmp, ct, rt, reinterpret_cast<float4 *>(W),
-                                                       reinterpret_cast<float2 *>(W_own));
+    launch_dependent(wind_gemm_kernel<T>, ct * rt, T * T / 64, 0, st, w, Lxy_t, lda, Btmp, ct, rt,
+                     reinterpret_cast<float4 *>(W), reinterpret_cast<float2 *>(W_own));
     count_launch();
     return cudaGetLastError();
 }
