@@ -54,7 +54,7 @@ typedef enum {
 #define TMA_MAX_AIRCRAFT 32          /* N: one warp lane per aircraft */
 #define TMA_MAX_PARTICLES (1 << 22)  /* L: keeps the fixed-point CDF products in 128 bits */
 #define TMA_MAX_GRID_Z 16
-#define TMA_MAX_GRAD_HORIZON 320     /* H of tma_rollout_grad: checkpoints kept per thread */
+#define TMA_MAX_GRAD_HORIZON 320     /* largest H of tma_rollout_grad */
 
 /* Move kinds of tma_set_move. */
 /* Bits of the sticky device error word (tma_get_error, tma_batch_results). */
@@ -300,10 +300,9 @@ tma_status tma_profile_read(tma_solver *s, tma_profile *h_out, int reset);
  * d_cbar_soft is not NULL, the per-aircraft means [N][L] (the same values as
  * tma_rollout_cost's soft means).  Reverse mode over the discrete dynamics of
  * Eq. (hor): limit, landing and interpolation-cell decisions are held at their
- * forward values; states are recomputed from checkpoints taken every 10
- * steps.  Valid for any sep_mode.  H must be <= TMA_MAX_GRAD_HORIZON
- * (TMA_ERR_UNSUPPORTED otherwise).  Uses solver-owned scratch, allocated on the
- * first call (not inside stream capture). */
+ * forward values.  Valid for any sep_mode.  H must be <= TMA_MAX_GRAD_HORIZON
+ * (TMA_ERR_UNSUPPORTED otherwise).  Uses solver-owned scratch (2 GB at most),
+ * allocated on the first call (not inside stream capture). */
 tma_status tma_rollout_grad(tma_solver *s, const float *d_u, int64_t L, int32_t J, float *d_cost,
                             float *d_grad, float *d_cbar_soft, tma_stream_t stream);
 

@@ -22,9 +22,9 @@
 //                         and fuel adjoints, and each segment's control gradient.
 // Limit, landing and interpolation-cell decisions keep their forward values.
 //
-// Bound: instruction issue (54 % busy, 780 warp instructions a step of 32 aircraft,
+// Bound: instruction issue (52 % busy, 750 warp instructions a step of 32 aircraft,
 // forward and back together; 1400 with the whole adjoint per sample) and the latency
-// of the wind gathers, here twice a step; DRAM 28 % for the sums and the flight log.
+// of the wind gathers, here twice a step; DRAM 31 % for the sums and the flight log.
 // Late particles, 12 aircraft, L 16384, M 16: 11.5 -> 7.3 ms; 24 aircraft, L 4096, M 8,
 // 90 steps: 6.05 -> 3.64 ms; 6 aircraft, L 4096, M 8: 0.67 -> 0.58 ms.  Of the 7.3 ms
 // the backward half is 3.2, the pairs 1.5, grad_controls_kernel 0.2.

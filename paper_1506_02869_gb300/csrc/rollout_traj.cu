@@ -24,10 +24,10 @@
 // that the costs are the one-sample tile's bits.
 //
 // Bound: the L1 data pipe (four 16-byte gathers of the wind cell a step) and
-// instruction issue, 78 and 65 % busy on the 8-aircraft workload.  Against the
+// instruction issue, 73-78 and 63-65 % busy on the 8-aircraft workload.  Against the
 // one-sample tile this drops from every sample's step the limit arithmetic, drag,
 // thrust, fuel, two compensated sums, the sine and cosine of the heading and the
-// vertical test of every pair (437 -> 262 warp instructions a step of 32
+// vertical test of every pair (437 -> 258 warp instructions a step of 32
 // aircraft, counted with 8 samples); it adds coalesced loads of 24 bytes a step.
 // Positions are exchanged once per four steps, nothing of the motion depends on
 // the partners.  Late particles: 8 aircraft, L 65536, M 32: 13.3 -> 9.4 ms; 24
