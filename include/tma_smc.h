@@ -166,8 +166,9 @@ tma_status tma_set_state(tma_solver *s, const tma_state *h_x0, uint32_t mpc_step
 
 /* Generate the solver's wind field for its current mpc_step (Sec. 3.9.1):
  * W(0) = Qhat v(0), W(k+1) = a W(k) + Q v(k+1) with Qhat = sigma (L_xy kron L_z),
- * Q = sqrt(1 - a^2) Qhat.  If d_W is not NULL the field is also copied there
- * (float32 [M][H][P][2]).  Uses solver-owned scratch. */
+ * Q = sqrt(1 - a^2) Qhat.  If d_W is not NULL the field is also written there
+ * (float32 [M][H][P][2]; any float-aligned address, TMA_ERR_INVALID_ARG
+ * otherwise).  Uses solver-owned scratch. */
 tma_status tma_wind_field(tma_solver *s, float *d_W, tma_stream_t stream);
 
 /* Random stream of the wind normals of this solver: 3 (default, the samples of

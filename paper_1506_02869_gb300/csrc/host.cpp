@@ -876,7 +876,7 @@ static tma_status gen_wind(tma_solver *s, cudaStream_t st, float *d_W)
 
 tma_status tma_wind_field(tma_solver *s, float *d_W, tma_stream_t stream)
 {
-    if (!s) return TMA_ERR_INVALID_ARG;
+    if (!s || reinterpret_cast<uintptr_t>(d_W) % alignof(float)) return TMA_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     return gen_wind(s, st, d_W);
 }

@@ -71,7 +71,7 @@ constexpr int kStages = 4, kKStep = 8;
 template <int T>
 __global__ void __launch_bounds__(T *T / 64, 6)
     wind_gemm_kernel(const WindC w, const float *__restrict__ At, int lda, const float *__restrict__ Bm, int n_ctiles,
-                     int n_rtiles, float4 *__restrict__ W, float2 *__restrict__ Wown)
+                     int n_rtiles, float4 *__restrict__ W, float *__restrict__ Wown, bool pairs)
 {
     constexpr int kThreads = T * T / 64, kPad = T + 2;   // rows an odd number of 8-byte words apart: no bank conflicts along rows
     constexpr int kRing = kStages * kKStep * 2 * T, kOut = 64 * kPad;
@@ -163,12 +163,19 @@ __global__ void __launch_bounds__(T *T / 64, 6)
             }
         }
         if (Wown) {
-            // the caller's layout [mk][row][level][2]: consecutive threads take consecutive levels
+            // the caller's layout [mk][row][level][2]: consecutive threads take consecutive
+            // levels; a pair in one store when the caller's pointer allows it
             for (int n = t; n < n_mk * rows * w.nz; n += kThreads) {
                 const int iz = n % w.nz, q = n / w.nz, mk = q / rows, r = q - mk * rows;
                 const float2 v = *reinterpret_cast<const float2 *>(sh + r * kPad + mk * two_nz + 2 * iz);
-                Wown[((size_t)(mk0 + mk) * w.nxy + r0 + r) * w.nz + iz] =
-                    make_float2(__fmul_rn(sg, v.x), __fmul_rn(sg, v.y));
+                float *o = Wown + 2 * (((size_t)(mk0 + mk) * w.nxy + r0 + r) * w.nz + iz);
+                const float2 own = make_float2(__fmul_rn(sg, v.x), __fmul_rn(sg, v.y));
+                if (pairs) {
+                    *reinterpret_cast<float2 *>(o) = own;
+                } else {
+                    o[0] = own.x;
+                    o[1] = own.y;
+                }
             }
         }
     }
@@ -199,7 +206,7 @@ cudaError_t launch_wind_gemm(const WindC &w, const float *Lxy_t, int lda, const 
     const int cols = wind_tile_cols(T, w.nz);
     const int ct = (w.ncol + cols - 1) / cols, rt = (w.nxy + T - 1) / T;
     launch_dependent(wind_gemm_kernel<T>, ct * rt, T * T / 64, 0, st, w, Lxy_t, lda, Btmp, ct, rt,
-                     reinterpret_cast<float4 *>(W), reinterpret_cast<float2 *>(W_own));
+                     reinterpret_cast<float4 *>(W), W_own, reinterpret_cast<uintptr_t>(W_own) % sizeof(float2) == 0);
     count_launch();
     return cudaGetLastError();
 }
