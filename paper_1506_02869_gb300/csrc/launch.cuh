@@ -1,13 +1,23 @@
 // Launches that overlap the previous kernel's end (programmatic dependent launch).
 //
 // A kernel launched by launch_dependent may be set up, its blocks placed, while the
-// kernel before it in the stream still runs; it begins with grid_begin, which lets the
-// next such kernel be set up and then waits until every kernel before it has completed
-// and its writes are visible.  Nothing of the previous kernels' memory is touched
+// kernel before it in the stream still runs; it begins with grid_begin, which waits
+// until every kernel before it has completed and its writes are visible, and then lets
+// the next such kernel be set up.  Nothing of the previous kernels' memory is touched
 // before that, so the order is the stream's; what is saved is the launch and the
 // prologue between two kernels, about 1.5 us each, which is what short solves are
 // made of.  After anything else in the stream (another launch, a copy) it is an
 // ordinary launch.
+//
+// The next kernel is let in after the wait and not before it: with a queue of passes,
+// kernels let in before it were placed three and four ahead, wherever the running ones
+// left room first, and then ran crowded on those SMs.  Calls one after the other, before
+// -> after: gradient of 8 aircraft, 60 steps, 1024 particles, one sample 238 -> 216 us,
+// of 2 aircraft, 30 steps, 4096 particles, 12 samples 198 -> 182 us; solve of 4 aircraft
+// with Langevin moves 560 -> 531 us, of 2 aircraft 462 -> 434 us.  grid_begin_early lets
+// it in before the wait: the last kernels of the resampling and of the selection, behind
+// which nothing crowds (the weights of 3 x 100000 particles 33.5 us without, 26.0 with it,
+// 26.5 with it in every kernel).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -17,6 +27,12 @@
 namespace tma {
 
 __device__ __forceinline__ void grid_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void grid_begin_early()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(kThreads) res_expand(const double *__restrict_
     __shared__ unsigned long long seg_before, seg_total;
     __shared__ Thresholds Tsh;
     __shared__ ChunkBase Bsh;
-    grid_begin();
+    grid_begin_early();
     const int s = blockIdx.y, c = blockIdx.x;
     const long long base = (long long)c * kChunk;
     const int len = (int)min((long long)kChunk, L - base);

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(256) select_final(const Cand *__restrict__ par
                                                     double *__restrict__ out_sum,
                                                     int *__restrict__ out_ninf)
 {
-    grid_begin();
+    grid_begin_early();
     Cand best{1 << 30, 0.0, 1ll << 62};
     for (int j = threadIdx.x; j < nparts; j += blockDim.x)
         if (better(part[j], best)) best = part[j];
