@@ -17,6 +17,7 @@
 //                         the block's samples (a block takes 32, 16 or 8 particles and a
 //                         range of the samples, one after the other: no atomics, a
 //                         fixed order);
+//   grad_sum_kernel       with few tiles or many ranges, their sums, a thread per element;
 //   grad_controls_kernel  the costs' means over the samples; once per particle:
 //                         backwards with the summed sources, the altitude, airspeed, heading
 //                         and fuel adjoints, and each segment's control gradient.
@@ -25,9 +26,13 @@
 // Bound: instruction issue (52 % busy, 750 warp instructions a step of 32 aircraft,
 // forward and back together; 1400 with the whole adjoint per sample) and the latency
 // of the wind gathers, here twice a step; DRAM 31 % for the sums and the flight log.
-// Late particles, 12 aircraft, L 16384, M 16: 11.5 -> 7.3 ms; 24 aircraft, L 4096, M 8,
-// 90 steps: 6.05 -> 3.64 ms; 6 aircraft, L 4096, M 8: 0.67 -> 0.58 ms.  Of the 7.3 ms
-// the backward half is 3.2, the pairs 1.5, grad_controls_kernel 0.2.
+// Late particles, 12 aircraft, L 16384, M 16: 11.5 -> 7.4 ms; 24 aircraft, L 4096, M 8,
+// 90 steps: 6.05 -> 3.64 ms; 6 aircraft, L 4096, M 8: 0.67 -> 0.53 ms.  Of the 7.4 ms
+// the backward half is 3.2, the pairs 1.5, grad_controls_kernel 0.2.  With few particles
+// the four chains of dependent steps are the time, and grad_controls_kernel must not add
+// waits for memory to them: summing the ranges inside it, four steps at a time, took 8
+// aircraft, 90 steps, L 200, M 40 from 457 us (one kernel, checkpoints) to 1250 us, the
+// sums by a kernel of their own and the fetch ahead to 431 us.
 #include "wind_rollout.cuh"
 
 namespace tma {
@@ -248,7 +253,10 @@ __global__ void __launch_bounds__(256, kMinBlocks)
                     dead ? __int_as_float(0x7f800000) : fmaf(P.mu_sep, q.soft, -logf(fmaxf(JT, 1e-30f)));
             cg = cost_grad(P, A, JT, ab, invM);
         }
-        if (dead || !exists) continue;             // an infeasible particle's gradient is zero
+        if (dead || !exists) {                     // an infeasible particle's gradient is zero
+            if (exists) R.bad[(size_t)tile * TP + j] = 1u;
+            continue;
+        }
         // the landing step itself has no terms, only the fuel burned up to it
         const int k_top = q.landed ? q.k_end - 1 : H;
         if (q.landed) {
@@ -375,14 +383,57 @@ __device__ __forceinline__ StepCoef step_coef(const ProblemC &P, const AircraftC
     return c;
 }
 
-// The sums of four steps are gathered at a time, their loads in flight together.
-template <int TP>
-__global__ void __launch_bounds__(256, 2) grad_controls_kernel(const ProblemC P, const DynState *__restrict__ dyn,
-                                                            const float *__restrict__ u, const TrajOut R,
-                                                            const GradScratch G, long long l_begin, long long l_end,
-                                                            int n_tiles, int n_ranges, const float *__restrict__ cost_ms,
-                                                            long long L, float *__restrict__ cost,
-                                                            float *__restrict__ grad, float *__restrict__ cbar)
+// Sums over the ranges of samples, into the first range's place: one thread per element
+// of a range (n of them, B threads a step), the ranges in order; an infeasible particle's
+// are left out.
+__global__ void __launch_bounds__(256) grad_sum_kernel(const ProblemC P, const GradScratch G,
+                                                       const unsigned *__restrict__ bad, unsigned n, int B, int tp,
+                                                       int n_ranges)
+{
+    grid_begin();
+    const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    const unsigned row = e / (unsigned)B, t = e - row * (unsigned)B;      // row = tile H + step
+    const unsigned tile = row / (unsigned)P.H, ac = t / (unsigned)tp;
+    if (bad[tile * (unsigned)tp + (t - ac * (unsigned)tp)] != 0u) return;
+    const bool arrival = P.ac[ac].type == 0;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    float lf = 0.0f;
+#pragma unroll 8
+    for (int c = 0; c < n_ranges; ++c) {
+        const float4 q = G.acc[(size_t)c * n + e];
+        a.x += q.x;
+        a.y += q.y;
+        a.z += q.z;
+        a.w += q.w;
+        if (arrival) lf += G.land[(size_t)c * n + e];
+    }
+    G.acc[e] = a;
+    if (arrival) G.land[e] = lf;
+    if (row == tile * (unsigned)P.H) {
+        const unsigned m = n / (unsigned)P.H, o = tile * (unsigned)B + t;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int c = 0; c < n_ranges; ++c) {
+            const float4 q = G.sums[(size_t)c * m + o];
+            s.x += q.x;
+            s.y += q.y;
+            s.z += q.z;
+        }
+        G.sums[o] = s;
+    }
+}
+
+// Ahead: four steps are fetched while the four after them are worked on, from sums over
+// all the samples (n_ranges 1): for grids that leave the chip idle, where waiting for each
+// four is the kernel's time.  Else the ranges are summed here, with twice the blocks
+// resident instead.
+template <int TP, bool Ahead>
+__global__ void __launch_bounds__(256, Ahead ? 1 : 2)
+    grad_controls_kernel(const ProblemC P, const DynState *__restrict__ dyn, const float *__restrict__ u, const TrajOut R,
+                         const GradScratch G, long long l_begin, long long l_end, int n_tiles, int n_ranges,
+                         const float *__restrict__ cost_ms, long long L, float *__restrict__ cost,
+                         float *__restrict__ grad, float *__restrict__ cbar)
 {
     constexpr int KC = 4;
     __shared__ float means[256];
@@ -437,39 +488,52 @@ __global__ void __launch_bounds__(256, 2) grad_controls_kernel(const ProblemC P,
     int seg = (int)((long long)(k_stop - 1) * P.S / H);                 // the segment of step k
     int k_seg = (int)(((long long)seg * H + P.S - 1) / P.S);            // and its first step
     float4 post = state[(size_t)(k_stop - 1) * B];                      // the state after step k
-    for (int kt = k_stop - 1; kt >= 0; kt -= KC) {
-        // four steps: the states before them and the sums over the ranges, all these
-        // loads in flight together (one after the other they are the kernel's time)
+    const float4 *acc = G.acc + (size_t)tile * H * B + t;
+    const float *land = G.land + (size_t)tile * H * B + t;
+    // four steps: the states before them and the sums over the ranges, all these
+    // loads in flight together (one after the other they are the kernel's time)
+    struct Steps {
         float4 pre[KC], a[KC];
         float lf[KC];
+    };
+    const auto fetch = [&](Steps &q, int kt) {
 #pragma unroll
         for (int e = 0; e < KC; ++e) {
             const int k = kt - e;
-            pre[e] = k > 0 ? state[(size_t)(k - 1) * B]
-                           : make_float4(dyn->x0[i][2], dyn->x0[i][3], 0.0f, dyn->x0[i][4]);
-            a[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-            lf[e] = 0.0f;
-        }
-#pragma unroll 2
-        for (int c = 0; c < n_ranges; ++c) {
-            const size_t o = ((size_t)c * n_tiles + tile) * H * B + t;
-#pragma unroll
-            for (int e = 0; e < KC; ++e) {
-                const float4 q = G.acc[o + (size_t)max(kt - e, 0) * B];
-                a[e].x += q.x;
-                a[e].y += q.y;
-                a[e].z += q.z;
-                a[e].w += q.w;
+            q.pre[e] = k > 0 ? state[(size_t)(k - 1) * B]
+                             : make_float4(dyn->x0[i][2], dyn->x0[i][3], 0.0f, dyn->x0[i][4]);
+            q.a[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+            q.lf[e] = 0.0f;
+            if constexpr (Ahead) {
+                q.a[e] = acc[(size_t)max(k, 0) * B];
+                if (A.type == 0) q.lf[e] = land[(size_t)max(k, 0) * B];
             }
         }
-        if (A.type == 0) {
+        if constexpr (!Ahead) {
+            const size_t range = (size_t)n_tiles * H * B;
 #pragma unroll 2
-            for (int c = 0; c < n_ranges; ++c) {
-                const size_t o = ((size_t)c * n_tiles + tile) * H * B + t;
+            for (int c = 0; c < n_ranges; ++c)
 #pragma unroll
-                for (int e = 0; e < KC; ++e) lf[e] += G.land[o + (size_t)max(kt - e, 0) * B];
+                for (int e = 0; e < KC; ++e) {
+                    const float4 v = acc[c * range + (size_t)max(kt - e, 0) * B];
+                    q.a[e].x += v.x;
+                    q.a[e].y += v.y;
+                    q.a[e].z += v.z;
+                    q.a[e].w += v.w;
+                }
+            if (A.type == 0) {
+#pragma unroll 2
+                for (int c = 0; c < n_ranges; ++c)
+#pragma unroll
+                    for (int e = 0; e < KC; ++e) q.lf[e] += land[c * range + (size_t)max(kt - e, 0) * B];
             }
         }
+    };
+    Steps now, next;
+    if constexpr (Ahead) fetch(now, k_stop - 1);
+    for (int kt = k_stop - 1; kt >= 0; kt -= KC) {
+        if constexpr (Ahead) fetch(next, kt - KC);
+        else fetch(now, kt);
 #pragma unroll
         for (int e = 0; e < KC; ++e) {
             const int k = kt - e;
@@ -482,26 +546,27 @@ __global__ void __launch_bounds__(256, 2) grad_controls_kernel(const ProblemC P,
                 --seg;
                 k_seg = (int)(((long long)seg * H + P.S - 1) / P.S);
             }
-            const StepCoef c = step_coef(P, A, pre[e].x, pre[e].y, pre[e].w, m0 - pre[e].z, __ldg(ul + 3 * seg),
-                                         __ldg(ul + 3 * seg + 1), __ldg(ul + 3 * seg + 2));
-            Z += a[e].z;
-            CH += a[e].w;
-            FF += lf[e];
+            const StepCoef c = step_coef(P, A, now.pre[e].x, now.pre[e].y, now.pre[e].w, m0 - now.pre[e].z,
+                                         __ldg(ul + 3 * seg), __ldg(ul + 3 * seg + 1), __ldg(ul + 3 * seg + 2));
+            Z += now.a[e].z;
+            CH += now.a[e].w;
+            FF += now.lf[e];
             if (A.type != 0) {
                 Z = fmaf(gB, sgnf(post.x - A.Z), Z);
                 V = fmaf(gC, sgnf(post.y - A.vD), V);
             }
-            const float proj = fmaf(c.cc, a[e].x, c.sc * a[e].y);      // along-track adjoint
+            const float proj = fmaf(c.cc, now.a[e].x, c.sc * now.a[e].y);      // along-track adjoint
             const float fe = FF * c.e;                                  // fuel adjoint times d F'/d T
             gw += fmaf(P.dt, CH, fe * c.wT);
             gh += P.dt * Z + c.hP * proj + fe * c.hT;
             ga += fmaf(P.dt, V, fe * c.aT);
             V += c.vP * proj + FF * c.vT;
-            CH += c.cP * fmaf(-c.sc, a[e].x, c.cc * a[e].y);
+            CH += c.cP * fmaf(-c.sc, now.a[e].x, c.cc * now.a[e].y);
             Z += fe * c.zT;
             FF -= fe * c.mT;
-            post = pre[e];
+            post = now.pre[e];
         }
+        if constexpr (Ahead) now = next;
     }
     gout[3 * seg] = gw;
     gout[3 * seg + 1] = gh;
@@ -512,7 +577,7 @@ __global__ void __launch_bounds__(256, 2) grad_controls_kernel(const ProblemC P,
 size_t grad_bytes(const ProblemC &P, size_t n, int n_ranges)
 {
     const size_t steps = n * (size_t)P.N * (size_t)P.H;
-    return traj_slab_bytes(P, n) + steps * sizeof(float4) +
+    return traj_slab_bytes(P, n) + steps * sizeof(float4) + n * sizeof(unsigned) +
            (size_t)n_ranges * (steps * (2 * sizeof(float4) + 2 * sizeof(float2) + sizeof(float)) +
                                n * (size_t)P.N * ((size_t)n_chunks(P.H) * sizeof(unsigned) + sizeof(float4)));
 }
@@ -530,6 +595,7 @@ GradScratch grad_places(const ProblemC &P, size_t n, int n_ranges, void *ws, Tra
     G.log.polar = G.log.xy + steps * n_ranges;
     G.land = reinterpret_cast<float *>(G.log.polar + steps * n_ranges);
     G.log.near = reinterpret_cast<unsigned *>(G.land + steps * n_ranges);
+    R.bad = G.log.near + ac * n_chunks(P.H) * n_ranges;
     return G;
 }
 
@@ -545,6 +611,16 @@ auto with_samples_kernel(int N, int variant, F f)
     if (tp == 32) return f(grad_samples_kernel<4, 32>);
     return tp == 16 ? f(grad_samples_kernel<4, 16>) : f(grad_samples_kernel<4, 8>);
 }
+
+// Where grad_controls_kernel takes sums over all the samples and fetches ahead (with the
+// sums inside it -> by grad_sum_kernel): below two tiles for each of 152 SMs, where nothing
+// else hides its waits (6 aircraft, 30 steps, L 4096, M 8: 397 -> 262 us; 2 aircraft, 20
+// steps, L 1024, M 8: 102 -> 51 us); with more tiles from four ranges on (12 aircraft, 60
+// steps, L 6000, M 16, four ranges: 2850 -> 2833 us; L 9000, three: 4339 -> 4356 us, not
+// taken).  Not for the shortest horizons: a range inside costs about 1 us per four steps,
+// the launch 4 us (1 aircraft, 5 steps, L 200, M 2: 28 against 30 us).
+constexpr int kFewTiles = 304;
+constexpr int kInlineSums = 4;     // fours of steps, times ranges beyond the first
 
 size_t samples_smem(int N) { return (size_t)wind_rollout_words(N, traj_tile(N), true, false) * sizeof(float); }
 
@@ -597,19 +673,36 @@ cudaError_t launch_rollout_grad(const ProblemC &P, const DynState *dyn, const fl
         const int n_tiles = (int)((l1 - l0 + tp - 1) / tp);
         launch_trajectories(P, dyn, u, l0, l1, R, true, st, true);
         with_samples_kernel(P.N, variant, [&](auto kernel) {
-            launch_dependent(kernel, (unsigned)n_tiles * (unsigned)n_ranges, block, smem, st, P, dyn, W4, R, G, L, l0, l1,
-                             n_tiles, m_per_block, J, cost_ms);
+            // one-warp blocks let in beside the trajectories were placed crowded: 1 aircraft,
+            // 30 steps, L 4096, M 12 106 us so, 82 us by an ordinary launch
+            const unsigned grid = (unsigned)n_tiles * (unsigned)n_ranges;
+            if (block > 32)
+                launch_dependent(kernel, grid, block, smem, st, P, dyn, W4, R, G, L, l0, l1, n_tiles, m_per_block, J,
+                                 cost_ms);
+            else
+                kernel<<<grid, block, smem, st>>>(P, dyn, W4, R, G, L, l0, l1, n_tiles, m_per_block, J, cost_ms);
             return 0;
         });
         count_launch();
         if (cost) {
-#define TMA_CONTROLS(TP)                                                                                              \
-    launch_dependent(grad_controls_kernel<TP>, n_tiles, block, 0, st, P, dyn, u, R, G, l0, l1, n_tiles, n_ranges,     \
-                     cost_ms, L, cost, grad, cbar)
-            if (tp == 32) TMA_CONTROLS(32);
-            else if (tp == 16) TMA_CONTROLS(16);
-            else TMA_CONTROLS(8);
-#undef TMA_CONTROLS
+            // few tiles, or many ranges: their sums by a kernel of its own
+            const bool sum = n_ranges > 1 && n_chunks(P.H) * (n_ranges - 1) > kInlineSums &&
+                             (n_tiles < kFewTiles || n_ranges > 3);
+            const int left = sum ? 1 : n_ranges;
+            if (sum) {
+                const unsigned elems = (unsigned)n_tiles * (unsigned)P.H * (unsigned)block;
+                launch_dependent(grad_sum_kernel, (elems + 255) / 256, 256, 0, st, P, G, R.bad, elems, block, tp,
+                                 n_ranges);
+                count_launch();
+            }
+            const auto controls = [&](auto kernel) {
+                launch_dependent(kernel, n_tiles, block, 0, st, P, dyn, u, R, G, l0, l1, n_tiles, left, cost_ms, L, cost,
+                                 grad, cbar);
+            };
+            const bool ahead = left == 1 && n_tiles < kFewTiles;
+            if (tp == 32) ahead ? controls(grad_controls_kernel<32, true>) : controls(grad_controls_kernel<32, false>);
+            else if (tp == 16) ahead ? controls(grad_controls_kernel<16, true>) : controls(grad_controls_kernel<16, false>);
+            else ahead ? controls(grad_controls_kernel<8, true>) : controls(grad_controls_kernel<8, false>);
             count_launch();
         }
         const cudaError_t e = cudaGetLastError();

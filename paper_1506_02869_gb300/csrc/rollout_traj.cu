@@ -66,6 +66,8 @@ __global__ void __launch_bounds__(256) trajectory_kernel(const ProblemC P, const
     const float reach = Soft ? P.sp_far_v : P.Sv;
     Kahan dB, dC;
     int kd = s.dead ? 0 : P.H;
+    if constexpr (States)
+        if (i == 0) R.bad[(size_t)blockIdx.x * TP + j] = exists ? 0u : 1u;
     size_t o = (size_t)blockIdx.x * P.H * B + t, om = (size_t)blockIdx.x * n_chunks(P.H) * B + t;
     constexpr int KB = kStepsPerBarrier;
     static_assert(KB == 4, "a chunk's masks are one uint4");
@@ -199,6 +201,7 @@ TrajOut traj_records(const ProblemC &P, size_t n, void *ws)
     TrajOut R;
     R.air = static_cast<float4 *>(ws);
     R.state = nullptr;
+    R.bad = nullptr;
     R.fin = R.air + n * P.N * (size_t)P.H;
     R.mask = reinterpret_cast<uint4 *>(R.fin + n * P.N);
     R.chi = reinterpret_cast<float *>(R.mask + n * P.N * (size_t)n_chunks(P.H));

@@ -16,6 +16,7 @@ struct TrajOut {
     float *fuel;       // arrivals: fuel burned after step k
     uint4 *mask;       // partner masks of the steps of chunk c: element ((tile nc + c) B + t), nc = ceil(H / 4)
     float4 *state;     // the gradient's: z, v, fuel burned, chi after step k (else nullptr)
+    unsigned *bad;     // the gradient's: [tile][TP], not 0: infeasible under some sample (else nullptr)
     float4 *fin;       // [tile][B]: sum |Z - z|, sum |v - vD|, fuel burned, stopping step (int; H: none)
 };
 
