@@ -302,8 +302,10 @@ tma_status tma_profile_read(tma_solver *s, tma_profile *h_out, int reset);
  * tma_rollout_cost's soft means).  Reverse mode over the discrete dynamics of
  * Eq. (hor): limit, landing and interpolation-cell decisions are held at their
  * forward values.  Valid for any sep_mode.  H must be <= TMA_MAX_GRAD_HORIZON
- * (TMA_ERR_UNSUPPORTED otherwise).  Uses solver-owned scratch (2 GB at most),
- * allocated on the first call (not inside stream capture). */
+ * (TMA_ERR_UNSUPPORTED otherwise).  Uses solver-owned scratch, allocated on the
+ * first call (not inside stream capture): 2 GB at most, 6 GB where few particles
+ * under many samples and a long horizon fill the device only so, and beyond 64 MB no
+ * more than a sixteenth of the free memory (what does not fit runs in slabs). */
 tma_status tma_rollout_grad(tma_solver *s, const float *d_u, int64_t L, int32_t J, float *d_cost,
                             float *d_grad, float *d_cbar_soft, tma_stream_t stream);
 

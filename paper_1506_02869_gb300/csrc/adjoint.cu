@@ -35,6 +35,8 @@
 // sums by a kernel of their own and the fetch ahead to 431 us.
 #include "wind_rollout.cuh"
 
+#include <algorithm>
+
 namespace tma {
 
 namespace {
@@ -573,7 +575,7 @@ __global__ void __launch_bounds__(256, Ahead ? 1 : 2)
     gout[3 * seg + 2] = ga;
 }
 
-// bytes of the scratch of n particles (a multiple of 32), and its places in a buffer
+// bytes of the scratch of n particles (a multiple of the tile), and its places in a buffer
 size_t grad_bytes(const ProblemC &P, size_t n, int n_ranges)
 {
     const size_t steps = n * (size_t)P.N * (size_t)P.H;
@@ -645,11 +647,28 @@ cudaError_t rollout_grad_occupancy(int N, int variant, int *blocks_per_sm)
 
 int rollout_grad_tile(int N) { return traj_tile(N); }
 
-size_t rollout_grad_workspace(const ProblemC &P, int64_t L, int n_ranges, size_t most)
+GradPlan rollout_grad_plan(const ProblemC &P, int64_t L, int n_ranges, int slots, size_t budget, size_t wide)
 {
-    const size_t per32 = grad_bytes(P, 32, n_ranges);
-    const size_t want = ((size_t)L + 31) / 32, fit = most / per32;
-    return (want < fit ? want : (fit > 0 ? fit : 1)) * per32;
+    const size_t tp = traj_tile(P.N), tiles = ((size_t)L + tp - 1) / tp;
+    const size_t base = grad_bytes(P, tp, 0), per = grad_bytes(P, tp, 1) - base;     // of a tile
+    const auto ranges_in = [&](size_t n) { return budget / n > base ? (budget / n - base) / per : 0; };
+    size_t r = (size_t)n_ranges, n = budget / (base + r * per);
+    if (n < tiles && n * r < (size_t)slots) {
+        // A slab with all the ranges would leave the chip idle (few particles, many
+        // samples, a long horizon): wide, or else fewer ranges for more tiles, but a
+        // resident wave of blocks if that fits.  32 aircraft, 320 steps, 512 samples:
+        // L 32 6.5 ms with all the ranges (5.3 GB), 8.5 ms with those of 2 GB.
+        if (tiles * (base + r * per) > wide) {
+            const size_t wave = std::min(r, ((size_t)slots + tiles - 1) / tiles);
+            r = std::max(std::min(r, ranges_in(tiles)), wave);
+            r = std::max(std::min(r, ranges_in(1)), (size_t)1);
+            n = budget / (base + r * per);
+        } else {
+            n = tiles;
+        }
+    }
+    n = std::min(std::max(n, (size_t)1), tiles);
+    return GradPlan{(int)r, n * (base + r * per)};
 }
 
 cudaError_t launch_rollout_grad(const ProblemC &P, const DynState *dyn, const float *u, const float *W, int64_t L,
@@ -659,13 +678,13 @@ cudaError_t launch_rollout_grad(const ProblemC &P, const DynState *dyn, const fl
     if (L <= 0) return cudaSuccess;
     const int m_per_block = (P.M + n_ranges - 1) / n_ranges;
     n_ranges = (P.M + m_per_block - 1) / m_per_block;
-    const size_t slab = ws_bytes / grad_bytes(P, 32, n_ranges) * 32, all = ((size_t)L + 31) / 32 * 32;
+    const int tp = traj_tile(P.N), block = P.N * tp;
+    const size_t slab = ws_bytes / grad_bytes(P, tp, n_ranges) * tp, all = ((size_t)L + tp - 1) / tp * tp;
     if (!ws || slab == 0) return cudaErrorInvalidValue;
     const size_t n = slab < all ? slab : all;
     TrajOut R;
     const GradScratch G = grad_places(P, n, n_ranges, ws, R);
     const float4 *W4 = reinterpret_cast<const float4 *>(W);
-    const int tp = traj_tile(P.N), block = P.N * tp;
     const size_t smem = samples_smem(P.N);
     const auto slab_end = [&](int64_t l0) { return l0 + (int64_t)n < L ? l0 + (int64_t)n : L; };
     for (int64_t l0 = 0; l0 < L; l0 += (int64_t)n) {

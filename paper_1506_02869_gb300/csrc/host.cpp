@@ -992,34 +992,50 @@ static int grad_chunks(tma_solver *s, int64_t L, int variant, int M)
     return (int)std::max(1LL, std::min<long long>(c, M));
 }
 
-static tma_status ensure_grad_scratch(tma_solver *s, int64_t L, int nchunk)
+// the gradient's scratch at most (larger calls run in slabs), and where that would leave the chip idle
+constexpr size_t kGradScratch = (size_t)2 << 30, kGradScratchWide = (size_t)6 << 30;
+
+// Scratch for a gradient of L particles, and the ranges of samples that it is made for.
+// The buffer is grown when a call wants more than any call before it; it is no more
+// than 64 MB or a sixteenth of the free memory, and when even that is not to be had,
+// half as much again and again, down to one tile in one range: such calls run in more
+// slabs or fewer ranges.
+static tma_status ensure_grad_scratch(tma_solver *s, int64_t L, int variant, int M, int *n_ranges)
 {
     const tma_problem &p = s->prob;
     if (!s->d_gcost_ms) {
         cudaError_t e = alloc(&s->d_gcost_ms, (size_t)p.M * p.N * p.L * sizeof(float));
         if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TMA_ERR_OOM : record_cuda_error(e);
     }
-    // 2 GB at most (larger particle counts run in slabs); on a nearly full device
-    // half as much again and again, down to the smallest slab
-    const ProblemC &P = s->P;
-    size_t want = rollout_grad_workspace(P, L, nchunk, (size_t)2 << 30);
-    const size_t asked = want, least = rollout_grad_workspace(P, 1, nchunk, 0);
-    if (want <= s->gwork_asked) return TMA_OK;
-    s->gwork_asked = 0;
-    if (s->d_gwork) cudaFree(s->d_gwork);
-    s->d_gwork = nullptr;
-    s->gwork_bytes = 0;
-    for (;;) {
-        const cudaError_t e = cudaMalloc(&s->d_gwork, want);
-        if (e == cudaSuccess) break;
+    const int wanted = grad_chunks(s, L, variant, M);
+    const auto plan_in = [&](size_t most) {
+        return rollout_grad_plan(s->P, L, wanted, s->grad_slots[variant], std::min(most, kGradScratch), most);
+    };
+    GradPlan plan = plan_in(kGradScratchWide);
+    if (plan.bytes > s->gwork_asked) {
+        const size_t asked = plan.bytes, least = plan_in(0).bytes;
+        if (s->d_gwork) cudaFree(s->d_gwork);
         s->d_gwork = nullptr;
-        if (e != cudaErrorMemoryAllocation) return record_cuda_error(e);
-        cudaGetLastError();
-        if (want <= least) return TMA_ERR_OOM;
-        want = std::max(least, want / 2);
+        s->gwork_bytes = s->gwork_asked = 0;
+        size_t budget = kGradScratchWide, free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess)
+            budget = std::min(budget, std::max((size_t)64 << 20, free_b / 16));
+        for (;;) {
+            plan = plan_in(budget);
+            const cudaError_t e = cudaMalloc(&s->d_gwork, plan.bytes);
+            if (e == cudaSuccess) break;
+            s->d_gwork = nullptr;
+            if (e != cudaErrorMemoryAllocation) return record_cuda_error(e);
+            cudaGetLastError();
+            if (plan.bytes <= least) return TMA_ERR_OOM;
+            budget = plan.bytes / 2;
+        }
+        s->gwork_bytes = plan.bytes;
+        s->gwork_asked = asked;
+    } else if (plan.bytes > s->gwork_bytes) {
+        plan = plan_in(s->gwork_bytes);            // the memory was short when it was taken
     }
-    s->gwork_bytes = want;
-    s->gwork_asked = asked;
+    *n_ranges = plan.n_ranges;
     return TMA_OK;
 }
 
@@ -1046,9 +1062,9 @@ static tma_status autotune_grad(tma_solver *s)
     }
     const int64_t Lp = std::min<int64_t>(s->prob.L, 4096);
     const size_t nu = (size_t)Lp * s->prob.N * s->prob.S * 3;
-    int max_chunks = 1;
-    for (int c = 0; c < nc; ++c) max_chunks = std::max(max_chunks, grad_chunks(s, Lp, cand[c], s->prob.M));
-    tma_status r = ensure_grad_scratch(s, Lp, max_chunks);
+    tma_status r = TMA_OK;
+    int nch = 1;
+    for (int c = 0; c < nc && r == TMA_OK; ++c) r = ensure_grad_scratch(s, Lp, cand[c], s->prob.M, &nch);
     if (r != TMA_OK) return r;
     cudaStream_t st = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1069,8 +1085,8 @@ static tma_status autotune_grad(tma_solver *s)
     if (e == cudaSuccess) e = launch_init_controls(s->P, s->d_dyn, lo, hi, d_u, Lp, st);
     float best = 1e30f;
     for (int c = 0; c < nc && e == cudaSuccess; ++c) {
-        const int nch = grad_chunks(s, Lp, cand[c], s->prob.M);
         // one untimed launch, then two timed
+        if ((r = ensure_grad_scratch(s, Lp, cand[c], s->prob.M, &nch)) != TMA_OK) break;
         e = launch_rollout_grad(s->P, s->d_dyn, d_u, s->d_W, Lp, 0, nch, s->d_gcost_ms, s->d_gwork,
                                 s->gwork_bytes, nullptr, nullptr, nullptr, st, cand[c]);
         if (e == cudaSuccess) e = cudaEventRecord(e0, st);
@@ -1111,8 +1127,8 @@ static tma_status grad_into(tma_solver *s, const float *d_u, int64_t L, int32_t 
     tma_status r = autotune_grad(s);
     if (r != TMA_OK) return r;
     const ProblemC Pj = problem_at(s, J);
-    const int nchunk = grad_chunks(s, L, s->grad_variant, Pj.M);
-    r = ensure_grad_scratch(s, L, nchunk);
+    int nchunk = 1;
+    r = ensure_grad_scratch(s, L, s->grad_variant, Pj.M, &nchunk);
     if (r != TMA_OK) return r;
     StageTimer t(s, 8, st);
     TMA_CUDA(launch_rollout_grad(Pj, s->d_dyn, d_u, s->d_W, L, J, nchunk, s->d_gcost_ms,
@@ -1199,7 +1215,8 @@ extern "C" tma_status tma_set_move(tma_solver *s, int32_t kind, double eps0)
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TMA_ERR_OOM : record_cuda_error(e);
     if (kind == TMA_MOVE_MALA) {
         r = autotune_grad(s);
-        if (r == TMA_OK) r = ensure_grad_scratch(s, p.L, grad_chunks(s, p.L, s->grad_variant, p.M));
+        int n_ranges = 1;
+        if (r == TMA_OK) r = ensure_grad_scratch(s, p.L, s->grad_variant, p.M, &n_ranges);
         if (r != TMA_OK) return r;
     }
     s->move_kind = kind;

@@ -196,15 +196,21 @@ cudaError_t launch_gather_best(const float *u, const int64_t *best, int nctl_per
                                float *best_u, cudaStream_t st, const unsigned int *flags = nullptr,
                                const int *ninf = nullptr, unsigned int *err = nullptr);
 
-// gradient of the soft cost (adjoint.cu): per-sample costs cost_ms[M][N][L]; ws: its
-// scratch, of which rollout_grad_workspace says how much L particles in n_ranges
-// ranges of samples want (at most `most`, but at least 32 particles' share: more run in
-// slabs); (cost == nullptr: the kernels over the samples only, for timing); variant
-// indexes the launch-bound table
+// gradient of the soft cost (adjoint.cu): per-sample costs cost_ms[M][N][L], samples in
+// n_ranges ranges; ws: its scratch, of which a tile's share in every range is the least
+// (more particles than it holds run in slabs); (cost == nullptr: the kernels over the
+// samples only, for timing); variant indexes the launch-bound table
 cudaError_t launch_rollout_grad(const ProblemC &P, const DynState *dyn, const float *u, const float *W, int64_t L,
                                 int J, int n_ranges, float *cost_ms, void *ws, size_t ws_bytes, float *cost, float *grad,
                                 float *cbar, cudaStream_t st, int variant);
-size_t rollout_grad_workspace(const ProblemC &P, int64_t L, int n_ranges, size_t most);
+// Ranges and scratch of a gradient of L particles within `budget` bytes (more only if the
+// least, one tile in one range, is more): n_ranges as asked while a slab then fills
+// `slots` resident blocks, else all the particles within `wide` bytes, or fewer ranges.
+struct GradPlan {
+    int n_ranges;
+    size_t bytes;
+};
+GradPlan rollout_grad_plan(const ProblemC &P, int64_t L, int n_ranges, int slots, size_t budget, size_t wide);
 cudaError_t rollout_grad_occupancy(int N, int variant, int *blocks_per_sm);
 int rollout_grad_variants(int N, int *out);
 int rollout_grad_tile(int N);      // particles per block
@@ -312,7 +318,7 @@ struct tma_solver {
     int *d_seg_scen1 = nullptr;
     // gradient scratch (allocated on first use)
     float *d_gcost_ms = nullptr;        // [M][N][L]
-    void *d_gwork = nullptr;            // the kernels' scratch (rollout_grad_workspace)
+    void *d_gwork = nullptr;            // the kernels' scratch (rollout_grad_plan)
     size_t gwork_bytes = 0, gwork_asked = 0;
     int grad_slots[8] = {0};            // resident blocks of each variant on the device (0: not asked yet)
     int grad_variant = -1;              // autotuned launch variant of the gradient kernel

@@ -323,7 +323,7 @@ __device__ __forceinline__ Flown wind_forward(const ProblemC &P, const DynState 
 int traj_tile(int N);
 void launch_trajectories(const ProblemC &P, const DynState *dyn, const float *u, long long l_begin, long long l_end,
                          const TrajOut &R, bool soft, cudaStream_t st, bool states = false);
-// The records' bytes for n particles (a multiple of 32) and their places in a buffer.
+// The records' bytes for n particles (a multiple of the tile) and their places in a buffer.
 size_t traj_slab_bytes(const ProblemC &P, size_t n);
 TrajOut traj_records(const ProblemC &P, size_t n, void *ws);
 
