@@ -477,10 +477,14 @@ static const uint32_t *dyn_mpc(const tma_solver *s)
 static std::mutex g_tune_mu;
 static std::map<std::string, int> g_tune_cache;
 
-static std::string tune_key_of(const tma_problem &p, int device)
+// The variants differ with the two-kernel form at hand or not (one sample, or no
+// workspace: a nearly full device): such solvers do not share their choice.
+static std::string tune_key_of(const tma_problem &p, const ProblemC &P, size_t traj_bytes, int device)
 {
     cudaDeviceProp prop;
     char key[320];
+    int tv[kMaxRolloutVariants];
+    const int two = rollout_traj_variants(P, traj_bytes, tv) > 0;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) prop.name[0] = 0;
     // the workload's size class: tiles of the tuning launch (32 particles x one
     // wind sample each, at most 8192 particles), by power of two -- a small
@@ -488,17 +492,17 @@ static std::string tune_key_of(const tma_problem &p, int device)
     const long long tiles = (std::min<long long>(p.L, 8192) + 31) / 32 * (long long)p.M;
     int lg = 0;
     while ((2LL << lg) <= tiles) ++lg;
-    snprintf(key, sizeof key, "%s|N=%d|pop=%d|wind=%d|rolling=%d|sep=%d|tiles=2^%d", prop.name, p.N,
-             p.pop_n[0] > 0, p.wind_mode, p.rolling, p.sep_mode, lg);
+    snprintf(key, sizeof key, "%s|N=%d|pop=%d|wind=%d|rolling=%d|sep=%d|tiles=2^%d|two=%d", prop.name, p.N,
+             p.pop_n[0] > 0, p.wind_mode, p.rolling, p.sep_mode, lg, two);
     return key;
 }
 
-static std::string tune_key(const tma_solver *s) { return tune_key_of(s->prob, s->device); }
+static std::string tune_key(const tma_solver *s) { return tune_key_of(s->prob, s->P, s->traj_bytes, s->device); }
 
-// Times every launch variant of the rollout kernel valid for P on the given
-// buffers (Lp particles, all wind samples, iteration 0, the soft costs too when
-// the problem has them): one untimed launch and three timed per variant; *best = the fastest, and the
-// timings in tv[] / tms[] (*nt entries).
+// Times the launch variants of the rollout that can be the fastest for P (the first
+// of rollout_variants) on the given buffers (Lp particles, all wind samples, iteration
+// 0, the soft costs too when the problem has them): one untimed launch and three timed
+// per variant; *best = the fastest, and the timings in tv[] / tms[] (*nt entries).
 static cudaError_t time_rollout_variants(const ProblemC &P, const DynState *dyn, const float *u,
                                          const float *W, int64_t Lp, float *cost, float *cost_soft, void *ws, size_t ws_bytes,
                                          cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int *best, int *nt, int *tv,
@@ -1819,7 +1823,7 @@ static tma_status batch_tune(tma_batch *b)
     // each scenario's best variant alone, and its best one of the one-sample kernel
     std::vector<int> one(n, 0);
     for (int s = 0; s < n && r == TMA_OK && e == cudaSuccess; ++s) {
-        const std::string key = tune_key_of(b->probs[s], b->device), key1 = key + "|one";
+        const std::string key = tune_key_of(b->probs[s], b->pc_h[s], b->traj_bytes, b->device), key1 = key + "|one";
         int best = -1;
         {
             std::lock_guard<std::mutex> g(g_tune_mu);

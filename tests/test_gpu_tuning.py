@@ -1,0 +1,34 @@
+"""The tuner's cache is shared by solvers with the same variants to choose from only."""
+import numpy as np
+import pytest
+
+import scenarios as S
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _solver(pkg, N, L, M):
+    rng = np.random.default_rng(N)
+    base = S.config5(n_scen=1)[0]
+    p = base.copy(N=N, L=L, M=M, H=12, grid=(5, 4, 3), sep_mode=2, aircraft=None)
+    p.aircraft = S._traffic(rng, (N + 1) // 2, N // 2, ring=45000.0, z_top=9000.0, sep_h=p.sep_h, sep_v=p.sep_v,
+                            dep_r=(2000.0, 30000.0))
+    return pkg.Solver(p)
+
+
+@pytest.mark.parametrize("N,order", [(26, (1, 2)), (22, (2, 1))])
+def test_one_sample_and_two_samples_of_one_size_class(N, order):
+    """One sample has no two-kernel variants; the same size class (tiles times samples) with two has.
+    (Kinds of problem that no other test tunes.)"""
+    import paper_1506_02869_gb300 as pkg
+    for M in order:
+        sol = _solver(pkg, N, 4096 // M, M)
+        variant, timed = pkg.tma_get_tuning(sol.h)
+        assert timed, M                                   # its own variants were timed, not another's choice taken
+        assert (18 in timed) == (M == 2), (M, timed)
+        pkg.tma_set_tuning(sol.h, variant)                # what was chosen can be chosen
+        sol.close()
+    again = _solver(pkg, N, 4096 // order[1], order[1])
+    assert not pkg.tma_get_tuning(again.h)[1]             # from the cache
+    again.close()
