@@ -510,7 +510,7 @@ static cudaError_t time_rollout_variants(const ProblemC &P, const DynState *dyn,
 {
     int cand[kMaxRolloutVariants];
     int nc = 0;
-    rollout_variants(P, ws_bytes, cand, &nc);
+    rollout_variants(P, ws_bytes, cand, &nc, Lp);
     *best = cand[0];
     *nt = 0;
     float best_ms = 1e30f;

@@ -95,7 +95,12 @@ constexpr int kPairCaps[] = {256, 256, 384, 512, 768};
 constexpr int kNumPairVariants = sizeof(kPairCaps) / sizeof(kPairCaps[0]);
 static_assert(kPairVariantBase + kNumPairVariants <= kHalfVariantBase, "variant table");
 
-int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed)
+// Threads (aircraft x particles x samples) up to which the smaller tiles are timed
+// beside the two-kernel form: about seven waves of 152 SMs with 1024 threads; creation
+// pays for each variant timed.
+constexpr long long kFewThreads = 1 << 20;
+
+int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed, int64_t L)
 {
     int n = 0, tv[kMaxRolloutVariants];
     const int nt = rollout_traj_variants(P, ws_bytes, tv);
@@ -108,11 +113,19 @@ int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed)
     // With the two-kernel form at hand the one-sample kernel is the faster one
     // only for small work (2 aircraft, 1024 particles, 8 samples: 23 against 33 us;
     // 32 aircraft, 200 particles, 8 samples: 196 on half tiles, 262 on whole ones),
-    // where its register budget and tile decide: one variant of each is timed.
+    // where its register budget and tile decide: one variant of each is timed, and up to
+    // a few waves of threads the smaller tiles too (soft forms of many aircraft: 28 aircraft,
+    // 223 particles, 12 samples 220 us with 1024-thread blocks, 207 on 8-particle tiles; 6215
+    // particles, 4 samples 7 % less on 16-particle ones).
     for (int c = 0; c < nt; ++c) out[n++] = kTrajVariantBase + tv[c];
     for (int v : {3, 7, 4})                      // 128, 85 and 64 registers
         if (nt > 0 && fits(v)) out[n++] = v;
     if (nt > 0 && small_tile_valid(P, 16, kHalfVariants[0].max_threads)) out[n++] = kHalfVariantBase;
+    if (nt > 0 && L > 0 && (long long)P.N * P.M * L <= kFewThreads) {
+        if (small_tile_valid(P, 16, kHalfVariants[2].max_threads)) out[n++] = kHalfVariantBase + 2;
+        for (int v = 0; v < kNumQuarterVariants; ++v)
+            if (small_tile_valid(P, 8, kQuarterVariants[v].max_threads)) out[n++] = kQuarterVariantBase + v;
+    }
     if (n_timed && nt > 0) *n_timed = n;
     for (int v = 0; v < kNumVariants; ++v)
         if (fits(v) && !listed(v)) out[n++] = v;
@@ -120,7 +133,8 @@ int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed)
         if (small_tile_valid(P, 16, kHalfVariants[v].max_threads) && !listed(kHalfVariantBase + v))
             out[n++] = kHalfVariantBase + v;
     for (int v = 0; v < kNumQuarterVariants; ++v)
-        if (small_tile_valid(P, 8, kQuarterVariants[v].max_threads)) out[n++] = kQuarterVariantBase + v;
+        if (small_tile_valid(P, 8, kQuarterVariants[v].max_threads) && !listed(kQuarterVariantBase + v))
+            out[n++] = kQuarterVariantBase + v;
     if (n_timed && nt == 0) *n_timed = n;
     if (nt > 0 && P.wind_mode == 0 && !P.rolling)
         for (int v = 0; v < kNumPairVariants; ++v)

@@ -153,8 +153,9 @@ cudaError_t launch_rollout(const ProblemC &P, const DynState *dyn, const float *
 // kQuarterVariantBase + v the one-sample kernel on 16- and 8-particle tiles,
 // kTrajVariantBase + v the two-kernel rollout of rollout_traj.cu, kPairVariantBase
 // + v the same under older names; returns their number (at least 1, at most
-// kMaxRolloutVariants).  The first n_timed are the ones the autotuner times.
-int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed = nullptr);
+// kMaxRolloutVariants).  The first n_timed are the ones the autotuner times for L
+// particles.
+int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed = nullptr, int64_t L = 0);
 // The two-kernel rollout: the workspace it wants (bytes, at most 512 MB: larger
 // particle counts run in slabs; 0 when the horizon is too long for it), its
 // variants (0-based) and its launcher.

@@ -1,4 +1,4 @@
-"""The tuner's cache is shared by solvers with the same variants to choose from only."""
+"""The tuner: what it times, and which solvers share a choice through its cache."""
 import numpy as np
 import pytest
 
@@ -32,3 +32,15 @@ def test_one_sample_and_two_samples_of_one_size_class(N, order):
     again = _solver(pkg, N, 4096 // order[1], order[1])
     assert not pkg.tma_get_tuning(again.h)[1]             # from the cache
     again.close()
+
+
+def test_small_work_times_the_smaller_tiles_too():
+    """Beside the two-kernel form the smaller tiles are the fastest for some small work; for large work
+    only the variants that can be are timed."""
+    import paper_1506_02869_gb300 as pkg
+    for L, M, small in ((223, 12, True), (8192, 64, False)):
+        sol = _solver(pkg, 28, L, M)
+        timed = pkg.tma_get_tuning(sol.h)[1]
+        assert {18, 19, 4, 13} <= set(timed), timed
+        assert ({15, 16, 17} <= set(timed)) == small, timed
+        sol.close()
