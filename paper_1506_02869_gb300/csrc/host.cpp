@@ -477,6 +477,15 @@ static const uint32_t *dyn_mpc(const tma_solver *s)
 static std::mutex g_tune_mu;
 static std::map<std::string, int> g_tune_cache;
 
+// Particles of the tuning launches: all, but at most 8192, or with few samples 131072
+// particle-samples.  (At 8192 of 20760 particles, 14 aircraft, 2 samples, the two-kernel
+// form was the faster one, 148 against 158 us; at all of them the one-sample kernel is,
+// 355 against 392 us.)
+static int64_t tuning_particles(const tma_problem &p)
+{
+    return std::min<int64_t>(p.L, std::max<int64_t>(8192, 131072 / p.M));
+}
+
 // The variants differ with the two-kernel form at hand or not (one sample, or no
 // workspace: a nearly full device): such solvers do not share their choice.
 static std::string tune_key_of(const tma_problem &p, const ProblemC &P, size_t traj_bytes, int device)
@@ -486,14 +495,17 @@ static std::string tune_key_of(const tma_problem &p, const ProblemC &P, size_t t
     int tv[kMaxRolloutVariants];
     const int two = rollout_traj_variants(P, traj_bytes, tv) > 0;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) prop.name[0] = 0;
-    // the workload's size class: tiles of the tuning launch (32 particles x one
-    // wind sample each, at most 8192 particles), by power of two -- a small
-    // solver's choice is not reused for a large one
-    const long long tiles = (std::min<long long>(p.L, 8192) + 31) / 32 * (long long)p.M;
-    int lg = 0;
-    while ((2LL << lg) <= tiles) ++lg;
-    snprintf(key, sizeof key, "%s|N=%d|pop=%d|wind=%d|rolling=%d|sep=%d|tiles=2^%d|two=%d", prop.name, p.N,
-             p.pop_n[0] > 0, p.wind_mode, p.rolling, p.sep_mode, lg, two);
+    // the workload's size class: tiles of the tuning launch (32 particles x one wind
+    // sample each) and wind samples (the two-kernel form shares a trajectory among
+    // them), by powers of two -- a small solver's choice is not reused for a large one
+    const auto class_of = [](long long n) {
+        int lg = 0;
+        while ((2LL << lg) <= n) ++lg;
+        return lg;
+    };
+    const int lg = class_of((tuning_particles(p) + 31) / 32 * (long long)p.M), lg_m = class_of(p.M);
+    snprintf(key, sizeof key, "%s|N=%d|pop=%d|wind=%d|rolling=%d|sep=%d|tiles=2^%d|M=2^%d|two=%d", prop.name,
+             p.N, p.pop_n[0] > 0, p.wind_mode, p.rolling, p.sep_mode, lg, lg_m, two);
     return key;
 }
 
@@ -814,8 +826,8 @@ tma_status tma_set_state(tma_solver *s, const tma_state *h_x0, uint32_t mpc_step
 static tma_status gen_wind(tma_solver *s, cudaStream_t st, float *d_W = nullptr);
 
 // Choose the rollout kernel's launch-bound variant by timing every valid
-// candidate on this solver's workload (uniform initial controls, at most 8192
-// particles, all wind samples); the choice is cached per device, aircraft
+// candidate on this solver's workload (uniform initial controls, tuning_particles,
+// all wind samples); the choice is cached per device, aircraft
 // count, problem kind and workload size class for the life of the process.
 static tma_status autotune_rollout(tma_solver *s)
 {
@@ -851,7 +863,7 @@ static tma_status autotune_rollout(tma_solver *s)
         return cuda_fail(e);
     }
     tma_status r = gen_wind(s, st);
-    const int64_t Lp = std::min<int64_t>(s->prob.L, 8192);
+    const int64_t Lp = tuning_particles(s->prob);
     float lo[3], hi[3], sg[3];
     ctrl_f(s->prob, lo, hi, sg);
     if (r == TMA_OK) {
@@ -1799,7 +1811,7 @@ static tma_status batch_solve_device(tma_batch *b, cudaStream_t st)
 
 // The batch's rollout dispatch: every scenario's variant of the single-scenario
 // kernel (the solvers' autotuner and cache, timed on the scenario's own first
-// 8192 particles), then both dispatch forms timed on the whole batch at
+// particles), then both dispatch forms timed on the whole batch at
 // iteration 0 (uniform initial controls; one untimed and one timed rollout
 // each); the faster form is kept.  On an idle device, like the solvers' tuner.
 static tma_status batch_tune(tma_batch *b)
@@ -1819,7 +1831,7 @@ static tma_status batch_tune(tma_batch *b)
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     tma_status r = e == cudaSuccess ? batch_wind(b, st) : cuda_fail(e);
     if (r == TMA_OK) e = launch_batch_init(b->d_scen, b->d_seg_scen, b->d_dyns, b->nseg, b->L, b->S, b->d_u[0], st);
-    const int64_t Lp = std::min<int64_t>(b->L, 8192);
+    const int64_t Lp = tuning_particles(b->probs[0]);
     // each scenario's best variant alone, and its best one of the one-sample kernel
     std::vector<int> one(n, 0);
     for (int s = 0; s < n && r == TMA_OK && e == cudaSuccess; ++s) {

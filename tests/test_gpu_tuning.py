@@ -44,3 +44,12 @@ def test_small_work_times_the_smaller_tiles_too():
         assert {18, 19, 4, 13} <= set(timed), timed
         assert ({15, 16, 17} <= set(timed)) == small, timed
         sol.close()
+
+
+def test_few_samples_of_many_particles_are_a_class_of_their_own():
+    """With two samples 32768 particles are tuned as such, not by the choice for 8192."""
+    import paper_1506_02869_gb300 as pkg
+    for L in (8192, 32768):
+        sol = _solver(pkg, 30, L, 2)
+        assert pkg.tma_get_tuning(sol.h)[1], L
+        sol.close()
