@@ -239,10 +239,11 @@ tma_status tma_get_particles(tma_solver *s, float *d_u_out, int64_t L, tma_strea
 tma_status tma_best_index(tma_solver *s, int64_t *h_best, tma_stream_t stream);
 
 /* Launch configuration of the rollout kernel chosen by the autotuner that
- * tma_create runs (Sec. 4.4 sweeps thread/block layouts by hand; here every
- * the launch-bound variants -- block-size cap and minimum resident blocks -- that
- * can be the fastest are timed on the solver's own workload and the fastest kept; the choice is
- * cached per device, aircraft count, problem kind and workload size class).
+ * tma_create runs (Sec. 4.4 sweeps thread/block layouts by hand; here the
+ * variants -- kernel form, block-size cap and minimum resident blocks -- that can be
+ * the fastest are timed on the solver's own workload and the fastest kept; the
+ * choice is cached per device, aircraft count, problem kind and workload size class,
+ * for solvers with the same variants to choose from).
  * *n_timed is 0 when the choice came from the cache; h_variants/h_ms (up to 24
  * entries, may be NULL) receive the
  * candidates and their mean time per rollout in ms. */
@@ -255,10 +256,12 @@ tma_status tma_get_tuning(tma_solver *s, int32_t *variant, int32_t *n_timed, int
  * 384x2, 768x1.  18-19: the two-kernel rollout (what does not depend on the wind
  * -- limits, drag, thrust, fuel, altitude, airspeed, heading, vertical
  * separation -- computed once per particle, the rest per sample), 256x4 and
- * 256x5, for M >= 2 and where memory for its workspace (at most 512 MB) was at
- * hand at creation.  8-12: older names of 18, for the shared wind field (wind
+ * 256x5, for M >= 2 and a solver that has its workspace: at most 512 MB, which must
+ * hold all particles or 1024 of them (32 aircraft: up to 585 steps beyond 1024
+ * particles) and, beyond 64 MB, be at most a sixteenth of the memory that was free at
+ * creation.  8-12: older names of 18, for M >= 2, the shared wind field (wind
  * mode 0) without the rolling window and block caps 256, 256, 384, 512, 768 at
- * 32 N threads.  13-15: the one-sample kernel on tiles of 16 particles (a
+ * 32 N threads; without the workspace they run the one-sample kernel.  13-15: the one-sample kernel on tiles of 16 particles (a
  * warp holds two aircraft; block 16 N threads), 768x1, 384x2, 512x2; 16-17: on
  * tiles of 8 particles (four aircraft per warp; block 8 N threads), 512x2,
  * 384x2; both for the shared wind field only and for N a multiple of 2 or 4

@@ -89,8 +89,9 @@ static bool small_tile_valid(const ProblemC &P, int tp, int cap)
 }
 
 // Variants 8-12, the names of an earlier kernel that computed the wind-independent
-// part once for two samples: they run the two-kernel form, for the problems and
-// block caps they always took (shared wind field, no rolling window).
+// part once for two samples: they run the two-kernel form (the one-sample kernel
+// without its workspace), for the problems and block caps they always took (shared
+// wind field, no rolling window, two samples).
 constexpr int kPairCaps[] = {256, 256, 384, 512, 768};
 constexpr int kNumPairVariants = sizeof(kPairCaps) / sizeof(kPairCaps[0]);
 static_assert(kPairVariantBase + kNumPairVariants <= kHalfVariantBase, "variant table");
@@ -136,7 +137,7 @@ int rollout_variants(const ProblemC &P, size_t ws_bytes, int *out, int *n_timed,
         if (small_tile_valid(P, 8, kQuarterVariants[v].max_threads) && !listed(kQuarterVariantBase + v))
             out[n++] = kQuarterVariantBase + v;
     if (n_timed && nt == 0) *n_timed = n;
-    if (nt > 0 && P.wind_mode == 0 && !P.rolling)
+    if (P.wind_mode == 0 && !P.rolling && P.M >= 2)
         for (int v = 0; v < kNumPairVariants; ++v)
             if (kPairCaps[v] >= P.N * kPB) out[n++] = kPairVariantBase + v;
     return n;

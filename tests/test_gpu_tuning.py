@@ -53,3 +53,26 @@ def test_few_samples_of_many_particles_are_a_class_of_their_own():
         sol = _solver(pkg, 30, L, 2)
         assert pkg.tma_get_tuning(sol.h)[1], L
         sol.close()
+
+
+def test_older_variant_names_without_a_workspace():
+    """8-12 are accepted for the problems they always were; where the two-kernel form has no workspace
+    (a long horizon beyond 1024 particles) they run the one-sample kernel: the same bits."""
+    import paper_1506_02869_gb300 as pkg
+    rng = np.random.default_rng(3)
+    base = S.config5(n_scen=1)[0]
+    p = base.copy(N=24, L=1056, M=2, H=900, grid=(4, 3, 2), sep_mode=0, aircraft=None)
+    p.aircraft = S._traffic(rng, 12, 12, ring=45000.0, z_top=9000.0, sep_h=p.sep_h, sep_v=p.sep_v, dep_r=(2000.0, 30000.0))
+    sol = pkg.Solver(p)
+    with pytest.raises(pkg.TmaError):
+        pkg.tma_set_tuning(sol.h, 18)
+    u = torch.from_numpy(S.mild_controls(p, p.L, rng) * np.float32(0.02)).cuda()
+    pkg.tma_set_tuning(sol.h, 4)
+    ref = sol.rollout_cost(u, 1)[0].clone()
+    assert bool(torch.isfinite(ref).any())
+    for v in (8, 11):
+        with pytest.raises(pkg.TmaError):                 # block caps of 256 and 512 threads
+            pkg.tma_set_tuning(sol.h, v)
+    pkg.tma_set_tuning(sol.h, 12)
+    assert torch.equal(sol.rollout_cost(u, 1)[0], ref)
+    sol.close()
