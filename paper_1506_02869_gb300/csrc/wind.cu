@@ -42,18 +42,24 @@ __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool on
                  : "memory");
 }
 
+// The product's tiles are kTile x kTile.
+constexpr int kTile = 64, kGemmThreads = kTile * kTile / 64;
+
 // Columns of a tile that are used: whole vertical columns of nodes (2 nz values
 // each, so that a node's upper neighbour is in the tile) and a multiple of 4
-// (16-byte copies).
-__host__ __device__ constexpr int wind_tile_cols(int T, int nz)
+// (16-byte copies).  All 64 for 2, 4, 8 and 16 levels, 36 for 9, 44 to 60 for the
+// others: the rest of such a tile's product is thrown away (64 x 64 x 9 grid, 4
+// samples, 30 steps: 1070 us, where 8 levels take 575; 1514 and 1375 us with the
+// 128 x 128 tiles that used every column).
+__host__ __device__ constexpr int wind_tile_cols(int nz)
 {
     const int unit = nz % 2 == 0 ? 2 * nz : 4 * nz;
-    return T / unit * unit;
+    return kTile / unit * unit;
 }
 
 // C[p][col] = sum_{q <= p} At[q][p] Btmp[q][col], q ascending in one chain of
-// fused multiply-adds per output, sigma C into the packed layout.  T x T tiles,
-// T = 64, 8 x 8 outputs per thread (64 threads: the two warps of a block wait for
+// fused multiply-adds per output, sigma C into the packed layout.  64 x 64 tiles,
+// 8 x 8 outputs per thread (64 threads: the two warps of a block wait for
 // little, and small fields fill the chip; 128 x 128 tiles of 256 threads were 8-30 %
 // slower from 5 samples of a 32 x 32 x 8 grid over 90 steps on), K in steps of 8
 // through a ring of four stages filled by cp.async; a pair of columns per
@@ -63,24 +69,24 @@ __host__ __device__ constexpr int wind_tile_cols(int T, int nz)
 // guards for the last columns only.  Row tiles run from the last (longest sums)
 // to the first.  Bound: the FP32 units (2.6e11 products and sums for 16 samples of
 // a 64 x 64 x 8 grid over 60 steps, 3.2 ms at their peak): that field with its
-// plain values takes 4.18 ms (normals included) against 9.47 ms with a
+// plain values takes 4.20 ms (normals included) against 9.47 ms with a
 // single-buffered loop, a second pass that formed the differences and a strided
 // copy for the plain values.
 constexpr int kStages = 4, kKStep = 8;
 
-template <int T>
-__global__ void __launch_bounds__(T *T / 64, 6)
+__global__ void __launch_bounds__(kGemmThreads, 6)
     wind_gemm_kernel(const WindC w, const float *__restrict__ At, int lda, const float *__restrict__ Bm, int n_ctiles,
                      int n_rtiles, float4 *__restrict__ W, float *__restrict__ Wown, bool pairs)
 {
-    constexpr int kThreads = T * T / 64, kPad = T + 2;   // rows an odd number of 8-byte words apart: no bank conflicts along rows
-    constexpr int kRing = kStages * kKStep * 2 * T, kOut = 64 * kPad;
+    constexpr int T = kTile, kThreads = kGemmThreads;
+    constexpr int kPad = T + 2;          // rows an odd number of 8-byte words apart: no bank conflicts along rows
+    constexpr int kRing = kStages * kKStep * 2 * T, kOut = T * kPad;
     __shared__ __align__(16) float sh[kRing > kOut ? kRing : kOut];
     grid_begin();
     const int t = threadIdx.x;
     const int tx = t % (T / 8), ty = t / (T / 8);
     const int rt = n_rtiles - 1 - (int)(blockIdx.x / n_ctiles);
-    const int cols = wind_tile_cols(T, w.nz);
+    const int cols = wind_tile_cols(w.nz);
     const int row0 = rt * T, col0 = (int)(blockIdx.x % n_ctiles) * cols;
     const int steps = (min(w.nxy, row0 + T) + kKStep - 1) / kKStep;
     float2 acc[8][4];
@@ -129,53 +135,49 @@ __global__ void __launch_bounds__(T *T / 64, 6)
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 
-    // through shared memory, 64 rows at a time, into the packed records: for each
-    // field mk and level, consecutive threads take consecutive rows (nodes along y)
+    // through shared memory into the packed records: for each field mk and level,
+    // consecutive threads take consecutive rows (nodes along y)
     const int two_nz = 2 * w.nz;
     const int mk0 = col0 / two_nz, n_mk = min(cols, w.ncol - col0) / two_nz;
     const float sg = w.sigma;
-    for (int h = 0; h < T / 64; ++h) {
-        __syncthreads();
-        if (ty / 8 == h) {
+    __syncthreads();
 #pragma unroll
-            for (int a = 0; a < 8; ++a) {
-                float2 *o = reinterpret_cast<float2 *>(sh + (ty % 8 * 8 + a) * kPad + tx * 4);
-                o[0] = acc[a][0];
-                o[1] = acc[a][1];
-                o[T / 4] = acc[a][2];
-                o[T / 4 + 1] = acc[a][3];
-            }
+    for (int a = 0; a < 8; ++a) {
+        float2 *o = reinterpret_cast<float2 *>(sh + (ty * 8 + a) * kPad + tx * 4);
+        o[0] = acc[a][0];
+        o[1] = acc[a][1];
+        o[T / 4] = acc[a][2];
+        o[T / 4 + 1] = acc[a][3];
+    }
+    __syncthreads();
+    const int rows = min(T, w.nxy - row0);
+    const int row = t % T, p = row0 + row;
+    if (row < rows) {
+        const size_t rec = (size_t)(p / w.ny) * w.out.pitch + p % w.ny;
+        const float *src = sh + row * kPad;
+        for (int c = t / T; c < n_mk * (w.nz - 1); c += kThreads / T) {
+            const int mk = c / (w.nz - 1), iz = c - mk * (w.nz - 1);
+            const float2 lo = *reinterpret_cast<const float2 *>(src + mk * two_nz + 2 * iz);
+            const float2 hi = *reinterpret_cast<const float2 *>(src + mk * two_nz + 2 * iz + 2);
+            const float2 own = make_float2(__fmul_rn(sg, lo.x), __fmul_rn(sg, lo.y));
+            W[(size_t)(mk0 + mk) * w.out.P + (size_t)iz * w.out.plane + rec] =
+                make_float4(own.x, own.y, __fsub_rn(__fmul_rn(sg, hi.x), own.x),
+                            __fsub_rn(__fmul_rn(sg, hi.y), own.y));
         }
-        __syncthreads();
-        const int r0 = row0 + h * 64, rows = min(64, w.nxy - r0);
-        const int row = t % 64, p = r0 + row;
-        if (row < rows) {
-            const size_t rec = (size_t)(p / w.ny) * w.out.pitch + p % w.ny;
-            const float *src = sh + row * kPad;
-            for (int c = t / 64; c < n_mk * (w.nz - 1); c += kThreads / 64) {
-                const int mk = c / (w.nz - 1), iz = c - mk * (w.nz - 1);
-                const float2 lo = *reinterpret_cast<const float2 *>(src + mk * two_nz + 2 * iz);
-                const float2 hi = *reinterpret_cast<const float2 *>(src + mk * two_nz + 2 * iz + 2);
-                const float2 own = make_float2(__fmul_rn(sg, lo.x), __fmul_rn(sg, lo.y));
-                W[(size_t)(mk0 + mk) * w.out.P + (size_t)iz * w.out.plane + rec] =
-                    make_float4(own.x, own.y, __fsub_rn(__fmul_rn(sg, hi.x), own.x),
-                                __fsub_rn(__fmul_rn(sg, hi.y), own.y));
-            }
-        }
-        if (Wown) {
-            // the caller's layout [mk][row][level][2]: consecutive threads take consecutive
-            // levels; a pair in one store when the caller's pointer allows it
-            for (int n = t; n < n_mk * rows * w.nz; n += kThreads) {
-                const int iz = n % w.nz, q = n / w.nz, mk = q / rows, r = q - mk * rows;
-                const float2 v = *reinterpret_cast<const float2 *>(sh + r * kPad + mk * two_nz + 2 * iz);
-                float *o = Wown + 2 * (((size_t)(mk0 + mk) * w.nxy + r0 + r) * w.nz + iz);
-                const float2 own = make_float2(__fmul_rn(sg, v.x), __fmul_rn(sg, v.y));
-                if (pairs) {
-                    *reinterpret_cast<float2 *>(o) = own;
-                } else {
-                    o[0] = own.x;
-                    o[1] = own.y;
-                }
+    }
+    if (Wown) {
+        // the caller's layout [mk][row][level][2]: consecutive threads take consecutive
+        // levels; a pair in one store when the caller's pointer allows it
+        for (int n = t; n < n_mk * rows * w.nz; n += kThreads) {
+            const int iz = n % w.nz, q = n / w.nz, mk = q / rows, r = q - mk * rows;
+            const float2 v = *reinterpret_cast<const float2 *>(sh + r * kPad + mk * two_nz + 2 * iz);
+            float *o = Wown + 2 * (((size_t)(mk0 + mk) * w.nxy + row0 + r) * w.nz + iz);
+            const float2 own = make_float2(__fmul_rn(sg, v.x), __fmul_rn(sg, v.y));
+            if (pairs) {
+                *reinterpret_cast<float2 *>(o) = own;
+            } else {
+                o[0] = own.x;
+                o[1] = own.y;
             }
         }
     }
@@ -202,10 +204,9 @@ cudaError_t launch_wind_normals_ar(const WindC &w, const DynState *dyn, float *B
 cudaError_t launch_wind_gemm(const WindC &w, const float *Lxy_t, int lda, const float *Btmp,
                              float *W, cudaStream_t st, float *W_own)
 {
-    constexpr int T = 64;
-    const int cols = wind_tile_cols(T, w.nz);
-    const int ct = (w.ncol + cols - 1) / cols, rt = (w.nxy + T - 1) / T;
-    launch_dependent(wind_gemm_kernel<T>, ct * rt, T * T / 64, 0, st, w, Lxy_t, lda, Btmp, ct, rt,
+    const int cols = wind_tile_cols(w.nz);
+    const int ct = (w.ncol + cols - 1) / cols, rt = (w.nxy + kTile - 1) / kTile;
+    launch_dependent(wind_gemm_kernel, ct * rt, kGemmThreads, 0, st, w, Lxy_t, lda, Btmp, ct, rt,
                      reinterpret_cast<float4 *>(W), W_own, reinterpret_cast<uintptr_t>(W_own) % sizeof(float2) == 0);
     count_launch();
     return cudaGetLastError();
