@@ -76,3 +76,32 @@ def test_older_variant_names_without_a_workspace():
     pkg.tma_set_tuning(sol.h, 12)
     assert torch.equal(sol.rollout_cost(u, 1)[0], ref)
     sol.close()
+
+
+def test_a_solver_without_room_for_the_workspace():
+    """On a nearly full device the two-kernel form's workspace is left out: the one-sample kernels run,
+    with the same bits, and a later solver of the same class has all its variants again."""
+    import paper_1506_02869_gb300 as pkg
+    ref = _solver(pkg, 14, 65536, 2)
+    assert 18 in pkg.tma_get_tuning(ref.h)[1]
+    g = torch.Generator(device="cuda").manual_seed(4)
+    u = 1e-3 * torch.randn((65536, 14, ref.S, 3), generator=g, device="cuda")
+    want = ref.rollout_cost(u, 1)[0].clone()
+    ref.close()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (3 << 29), dtype=torch.uint8, device="cuda")
+    sol = _solver(pkg, 14, 65536, 2)
+    timed = pkg.tma_get_tuning(sol.h)[1]
+    with pytest.raises(pkg.TmaError):
+        pkg.tma_set_tuning(sol.h, 18)
+    got = sol.rollout_cost(u, 1)[0].clone()
+    sol.close()
+    del hold
+    torch.cuda.empty_cache()
+    assert timed and not {18, 19} & set(timed)
+    assert bool(torch.isfinite(want).any()) and torch.equal(got, want)
+    again = _solver(pkg, 14, 65536, 2)
+    pkg.tma_set_tuning(again.h, 18)
+    assert torch.equal(again.rollout_cost(u, 1)[0], want)
+    again.close()
