@@ -106,23 +106,28 @@ def flops_per_unit_tally(p):
         pair * (p.N - 1) / 2.0
 
 
-# DRAM bytes (read + write) of one full-size rollout launch per workload and
-# rollout kernel, from a one-pass ncu capture (dram__bytes_read.sum +
-# dram__bytes_write.sum of one launch late in a solve: iteration 20 of 30);
-# valid only for the kernel sources they were taken on.
-ROLLOUT_TRAFFIC = {"sources_sha256_16": "9c6681ad7c36f584",
-                   "bytes_per_launch": {"c3:rollout_kernel": 47479898368 + 4464612352}}
+# DRAM bytes (read + write) of one full-size rollout (all launches of it) per
+# workload and rollout kernels, from a one-pass ncu capture (dram__bytes_read.sum +
+# dram__bytes_write.sum, late in a solve: iteration 20 of 30); valid only for the
+# kernel sources they were taken on.
+ROLLOUT_TRAFFIC = {"sources_sha256_16": "bdc1343cbe6d485d",
+                   "bytes_per_launch": {"c3:trajectory_kernel+wind_rollout_kernel": 1613256767232 + 19068303104}}
 
 
 def rollout_kernel_name(variant):
-    """The rollout kernel a launch variant runs (8-12 and 18-19: the two-kernel form; 13-15 and
-    16-17 the one-sample kernel on 16- and 8-particle tiles)."""
-    return "wind_rollout_kernel" if variant is not None and (8 <= variant < 13 or variant >= 18) else "rollout_kernel"
+    """The kernels of a rollout by a launch variant (8-12 and 18-19: the two-kernel form, a pair of
+    launches per slab of particles; 13-15 and 16-17 the one-sample kernel on 16- and 8-particle tiles)."""
+    return ("trajectory_kernel+wind_rollout_kernel" if variant is not None and (8 <= variant < 13 or variant >= 18)
+            else "rollout_kernel")
+
+
+ROLLOUT_SOURCES = ("rollout.cu", "rollout_traj.cu", "wind_rollout.cuh", "rollout_tile.cuh", "device_common.cuh",
+                   "launch.cuh", "tma_internal.h")
 
 
 def rollout_sources_digest():
     h = hashlib.sha256()
-    for f in ("rollout.cu", "rollout_traj.cu", "rollout_tile.cuh", "device_common.cuh"):
+    for f in ROLLOUT_SOURCES:
         with open(os.path.join(ROOT, "paper_1506_02869_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -211,11 +211,15 @@ TrajOut traj_records(const ProblemC &P, size_t n, void *ws)
 
 size_t traj_workspace(const ProblemC &P, int64_t L)
 {
-    // 24-256 MB slabs ran 10-2 % slower than 1 GB ones on 65536 particles of 8 aircraft
+    // 65536 particles of 8 aircraft, 32 samples: slabs of 24 MB 11.7 ms, 64-256 MB 10.5,
+    // 512 MB 10.32, 1 GB 10.24
     const size_t most = (size_t)512 << 20;
     const size_t per32 = traj_slab_bytes(P, 32);
     const size_t want = ((size_t)L + 31) / 32, fit = most / per32;
-    // a slab of few tiles would leave the chip idle: no workspace, one-sample kernels
+    // A slab of fewer than 1024 particles would leave the chip idle: no workspace,
+    // one-sample kernels.  (Long horizons: 32 aircraft beyond 584 steps.  With slabs of
+    // 1024 they ran 6.1 -> 4.6 ms, hard, but 6.4 -> 7.1 ms, soft, and 12.3 -> 12.9 ms of
+    // 8192 particles: the tuner's short first-iteration flights favour the two-kernel form.)
     if (fit < want && fit < 32) return 0;
     return (want < fit ? want : fit) * per32;
 }
