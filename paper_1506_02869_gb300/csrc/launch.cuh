@@ -14,10 +14,14 @@
 // left room first, and then ran crowded on those SMs.  Calls one after the other, before
 // -> after: gradient of 8 aircraft, 60 steps, 1024 particles, one sample 238 -> 216 us,
 // of 2 aircraft, 30 steps, 4096 particles, 12 samples 198 -> 182 us; solve of 4 aircraft
-// with Langevin moves 560 -> 531 us, of 2 aircraft 462 -> 434 us.  grid_begin_early lets
-// it in before the wait: the last kernels of the resampling and of the selection, behind
-// which nothing crowds (the weights of 3 x 100000 particles 33.5 us without, 26.0 with it,
-// 26.5 with it in every kernel).
+// with Langevin moves 560 -> 510 us, of 2 aircraft 459 -> 438 us.
+//
+// grid_begin_early lets it in before the wait: the short kernels between two rollouts
+// (sample means, normalisation, resampling) and the last one of the selection, which
+// are set up while a long rollout ends and behind which nothing crowds.  Without it for
+// them: solve of 8 aircraft, 60 steps, 4096 particles, 16 samples 2925 -> 3045 us, with
+// random-walk moves of 6 aircraft 1387 -> 1432 us, weights of 3 x 100000 particles 26.0
+// -> 33.5 us; in the moves and the two rollout kernels too it gained nothing.
 #pragma once
 
 #include <cuda_runtime.h>

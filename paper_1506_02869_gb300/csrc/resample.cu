@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kThreads) lse_chunk_min(const float *__restric
                                                           int nchunk, float *__restrict__ cmin)
 {
     __shared__ float sh[32];
-    grid_begin();
+    grid_begin_early();
     const int s = blockIdx.y, c = blockIdx.x;
     const float *row = cbar + (size_t)s * L;
     const long long base = (long long)c * kChunk;
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kThreads) lse_exp(const float *__restrict__ cb
     __shared__ unsigned long long tab[256];
     const int s = blockIdx.y, c = blockIdx.x;
     for (int j = threadIdx.x; j < 256; j += kThreads) tab[j] = kExp2Frac63[j];      // constants of the library
-    grid_begin();
+    grid_begin_early();
     float mn = __int_as_float(0x7f800000);
     for (int j = threadIdx.x; j < nchunk; j += kThreads) mn = fminf(mn, cmin[(size_t)s * nchunk + j]);
     mn = block_reduce(mn, MinOp(), shf, __int_as_float(0x7f800000));   // its barriers also cover tab
@@ -263,7 +263,7 @@ __global__ void lse_finish(const float *__restrict__ cmin, const double *__restr
                            int nchunk, double kappa, double *__restrict__ lmax,
                            double *__restrict__ wsum)
 {
-    grid_begin();
+    grid_begin_early();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nseg) return;
     float mn = __int_as_float(0x7f800000);
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kThreads) res_chunk_sum(const double *__restri
                                                           unsigned long long *__restrict__ cq)
 {
     __shared__ unsigned long long sh[32];
-    grid_begin();
+    grid_begin_early();
     const int s = blockIdx.y, c = blockIdx.x;
     const double *row = wtilde + (size_t)s * L;
     const long long base = (long long)c * kChunk;

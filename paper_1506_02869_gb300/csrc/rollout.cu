@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) sample_mean_kernel(const float *__restric
                                                           long long L, int M, int N,
                                                           float *__restrict__ cbar)
 {
-    grid_begin();
+    grid_begin_early();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L * N) return;
     Kahan s;
