@@ -515,14 +515,16 @@ static std::string tune_key(const tma_solver *s) { return tune_key_of(s->prob, s
 // of rollout_variants) on the given buffers (Lp particles, all wind samples, iteration
 // 0, the soft costs too when the problem has them): one untimed launch and three timed
 // per variant; *best = the fastest, and the timings in tv[] / tms[] (*nt entries).
+// alone: the device is this problem's (not a batch's, beside whose other scenarios the
+// smaller tiles, which fill an idle chip, are the slower ones).
 static cudaError_t time_rollout_variants(const ProblemC &P, const DynState *dyn, const float *u,
-                                         const float *W, int64_t Lp, float *cost, float *cost_soft, void *ws, size_t ws_bytes,
+                                         const float *W, int64_t Lp, bool alone, float *cost, float *cost_soft, void *ws, size_t ws_bytes,
                                          cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int *best, int *nt, int *tv,
                                          float *tms)
 {
     int cand[kMaxRolloutVariants];
     int nc = 0;
-    rollout_variants(P, ws_bytes, cand, &nc, Lp);
+    rollout_variants(P, ws_bytes, cand, &nc, alone ? Lp : 0);
     *best = cand[0];
     *nt = 0;
     float best_ms = 1e30f;
@@ -869,7 +871,7 @@ static tma_status autotune_rollout(tma_solver *s)
     if (r == TMA_OK) {
         e = launch_init_controls(s->P, s->d_dyn, lo, hi, s->d_u[0], Lp, st);
         if (e == cudaSuccess)
-            e = time_rollout_variants(s->P, s->d_dyn, s->d_u[0], s->d_W, Lp, s->d_cost_ms, s->d_cost_ms_soft,
+            e = time_rollout_variants(s->P, s->d_dyn, s->d_u[0], s->d_W, Lp, true, s->d_cost_ms, s->d_cost_ms_soft,
                                       s->d_traj, s->traj_bytes, st, e0, e1, &s->rollout_variant, &s->n_tuned, s->tuned_variant, s->tuned_ms);
         if (e != cudaSuccess) r = cuda_fail(e);
     }
@@ -1810,8 +1812,8 @@ static tma_status batch_solve_device(tma_batch *b, cudaStream_t st)
 }
 
 // The batch's rollout dispatch: every scenario's variant of the single-scenario
-// kernel (the solvers' autotuner and cache, timed on the scenario's own first
-// particles), then both dispatch forms timed on the whole batch at
+// kernel (timed as the solvers' is, on the scenario's own first particles, with
+// entries of its own in the cache), then both dispatch forms timed on the whole batch at
 // iteration 0 (uniform initial controls; one untimed and one timed rollout
 // each); the faster form is kept.  On an idle device, like the solvers' tuner.
 static tma_status batch_tune(tma_batch *b)
@@ -1835,7 +1837,8 @@ static tma_status batch_tune(tma_batch *b)
     // each scenario's best variant alone, and its best one of the one-sample kernel
     std::vector<int> one(n, 0);
     for (int s = 0; s < n && r == TMA_OK && e == cudaSuccess; ++s) {
-        const std::string key = tune_key_of(b->probs[s], b->pc_h[s], b->traj_bytes, b->device), key1 = key + "|one";
+        const std::string key = tune_key_of(b->probs[s], b->pc_h[s], b->traj_bytes, b->device) + "|batch";
+        const std::string key1 = key + "|one";
         int best = -1;
         {
             std::lock_guard<std::mutex> g(g_tune_mu);
@@ -1851,7 +1854,7 @@ static tma_status batch_tune(tma_batch *b)
         int fastest = 0, nt = 0, tv[kMaxRolloutVariants];
         float tms[kMaxRolloutVariants];
         e = time_rollout_variants(b->pc_h[s], b->d_dyns + s, b->d_u[0] + sc.u_off, b->d_W + (size_t)sc.w_off * 4,
-                                  Lp, b->d_cost_ms + (size_t)sc.seg_off * b->M * (size_t)b->L,
+                                  Lp, false, b->d_cost_ms + (size_t)sc.seg_off * b->M * (size_t)b->L,
                                   b->d_cost_ms_soft ? b->d_cost_ms_soft + (size_t)sc.seg_off * b->M * (size_t)b->L : nullptr,
                                   b->d_traj, b->traj_bytes, st, e0, e1, &fastest, &nt, tv, tms);
         if (e == cudaSuccess) {
