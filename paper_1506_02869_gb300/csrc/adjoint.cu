@@ -385,44 +385,63 @@ __device__ __forceinline__ StepCoef step_coef(const ProblemC &P, const AircraftC
     return c;
 }
 
-// Sums over the ranges of samples, into the first range's place: one thread per element
-// of a range (n of them, B threads a step), the ranges in order; an infeasible particle's
-// are left out.
+// Sums over the ranges of samples, into the first range's place: one thread per KS steps
+// of a (tile, thread t of B), the ranges in order; an infeasible particle's are left out.
+// Four steps a thread where one would be more threads than the chip holds: a quarter of
+// the blocks to start, and of those that find their particles infeasible.
+template <int KS>
 __global__ void __launch_bounds__(256) grad_sum_kernel(const ProblemC P, const GradScratch G,
-                                                       const unsigned *__restrict__ bad, unsigned n, int B, int tp,
-                                                       int n_ranges)
+                                                       const unsigned *__restrict__ bad, unsigned threads, int n_tiles,
+                                                       int B, int tp, int n_ranges)
 {
     grid_begin();
     const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const unsigned row = e / (unsigned)B, t = e - row * (unsigned)B;      // row = tile H + step
-    const unsigned tile = row / (unsigned)P.H, ac = t / (unsigned)tp;
+    if (e >= threads) return;
+    const unsigned row = e / (unsigned)B, t = e - row * (unsigned)B;
+    const unsigned per = (unsigned)(P.H + KS - 1) / KS, tile = row / per, k0 = (row - tile * per) * KS;
+    const unsigned ac = t / (unsigned)tp;
     if (bad[tile * (unsigned)tp + (t - ac * (unsigned)tp)] != 0u) return;
     const bool arrival = P.ac[ac].type == 0;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    float lf = 0.0f;
-#pragma unroll 8
-    for (int c = 0; c < n_ranges; ++c) {
-        const float4 q = G.acc[(size_t)c * n + e];
-        a.x += q.x;
-        a.y += q.y;
-        a.z += q.z;
-        a.w += q.w;
-        if (arrival) lf += G.land[(size_t)c * n + e];
+    const size_t range = (size_t)n_tiles * P.H * B;
+    const size_t o = ((size_t)tile * P.H + k0) * B + t;
+    const int steps = min(KS, P.H - (int)k0);
+    float4 a[KS];
+    float lf[KS];
+#pragma unroll
+    for (int q = 0; q < KS; ++q) {
+        a[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        lf[q] = 0.0f;
     }
-    G.acc[e] = a;
-    if (arrival) G.land[e] = lf;
-    if (row == tile * (unsigned)P.H) {
-        const unsigned m = n / (unsigned)P.H, o = tile * (unsigned)B + t;
+#pragma unroll(KS == 1 ? 8 : 2)
+    for (int c = 0; c < n_ranges; ++c) {
+#pragma unroll
+        for (int q = 0; q < KS; ++q) {
+            const size_t at = c * range + o + (size_t)min(q, steps - 1) * B;
+            const float4 v = G.acc[at];
+            a[q].x += v.x;
+            a[q].y += v.y;
+            a[q].z += v.z;
+            a[q].w += v.w;
+            if (arrival) lf[q] += G.land[at];
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < KS; ++q) {
+        if (q >= steps) break;
+        G.acc[o + (size_t)q * B] = a[q];
+        if (arrival) G.land[o + (size_t)q * B] = lf[q];
+    }
+    if (k0 == 0) {
+        const unsigned so = tile * (unsigned)B + t;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
         for (int c = 0; c < n_ranges; ++c) {
-            const float4 q = G.sums[(size_t)c * m + o];
+            const float4 q = G.sums[(size_t)c * n_tiles * B + so];
             s.x += q.x;
             s.y += q.y;
             s.z += q.z;
         }
-        G.sums[o] = s;
+        G.sums[so] = s;
     }
 }
 
@@ -622,6 +641,7 @@ auto with_samples_kernel(int N, int variant, F f)
 // taken).  Not for the shortest horizons: a range inside costs about 1 us per four steps,
 // the launch 4 us (1 aircraft, 5 steps, L 200, M 2: 28 against 30 us).
 constexpr int kFewTiles = 304;
+constexpr size_t kManyThreads = 152 * 2048;    // grad_sum_kernel: those of a step a thread that the chip holds
 constexpr int kInlineSums = 4;     // fours of steps, times ranges beyond the first
 
 size_t samples_smem(int N) { return (size_t)wind_rollout_words(N, traj_tile(N), true, false) * sizeof(float); }
@@ -709,9 +729,13 @@ cudaError_t launch_rollout_grad(const ProblemC &P, const DynState *dyn, const fl
                              (n_tiles < kFewTiles || n_ranges > 3);
             const int left = sum ? 1 : n_ranges;
             if (sum) {
-                const unsigned elems = (unsigned)n_tiles * (unsigned)P.H * (unsigned)block;
-                launch_dependent(grad_sum_kernel, (elems + 255) / 256, 256, 0, st, P, G, R.bad, elems, block, tp,
-                                 n_ranges);
+                const auto sums = [&](auto kernel, int ks) {
+                    const unsigned threads = (unsigned)n_tiles * (unsigned)((P.H + ks - 1) / ks) * (unsigned)block;
+                    launch_dependent(kernel, (threads + 255) / 256, 256, 0, st, P, G, R.bad, threads, n_tiles, block, tp,
+                                     n_ranges);
+                };
+                if ((size_t)n_tiles * P.H * block <= kManyThreads) sums(grad_sum_kernel<1>, 1);
+                else sums(grad_sum_kernel<4>, 4);
                 count_launch();
             }
             const auto controls = [&](auto kernel) {

@@ -27,7 +27,7 @@ def _problem(N, M, H, L):
 
 # samples capped so that few and many tiles split them alike: one a range
 @pytest.mark.parametrize("N,M,H", [(1, 9, 21), (1, 2, 5), (2, 1, 4), (3, 6, 21), (3, 2, 9), (8, 1, 33), (9, 2, 21), (9, 1, 7),
-                                   (17, 2, 22), (32, 2, 17), (32, 1, 1)])
+                                   (17, 2, 22), (32, 2, 17), (32, 1, 1), (8, 3, 50), (12, 2, 63)])
 def test_every_form_of_the_sums_returns_the_same_bits(N, M, H):
     import paper_1506_02869_gb300 as pkg
     tp = 32 if N <= 8 else (16 if N <= 16 else 8)
