@@ -110,8 +110,8 @@ def flops_per_unit_tally(p):
 # workload and rollout kernels, from a one-pass ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum, late in a solve: iteration 20 of 30); valid only for the
 # kernel sources they were taken on.
-ROLLOUT_TRAFFIC = {"sources_sha256_16": "bdc1343cbe6d485d",
-                   "bytes_per_launch": {"c3:trajectory_kernel+wind_rollout_kernel": 1613256767232 + 19068303104}}
+ROLLOUT_TRAFFIC = {"sources_sha256_16": "d0fddb37bc78b44c",
+                   "bytes_per_launch": {"c3:trajectory_kernel+wind_rollout_kernel": 1635639205888 + 19065694720}}
 
 
 def rollout_kernel_name(variant):

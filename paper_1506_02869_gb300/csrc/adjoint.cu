@@ -27,12 +27,12 @@
 // forward and back together; 1400 with the whole adjoint per sample) and the latency
 // of the wind gathers, here twice a step; DRAM 31 % for the sums and the flight log.
 // Late particles, 12 aircraft, L 16384, M 16: 11.5 -> 7.4 ms; 24 aircraft, L 4096, M 8,
-// 90 steps: 6.05 -> 3.64 ms; 6 aircraft, L 4096, M 8: 0.67 -> 0.53 ms.  Of the 7.4 ms
+// 90 steps: 6.13 -> 3.64 ms; 6 aircraft, L 4096, M 8: 0.66 -> 0.52 ms.  Of the 7.4 ms
 // the backward half is 3.2, the pairs 1.5, grad_controls_kernel 0.2.  With few particles
 // the four chains of dependent steps are the time, and grad_controls_kernel must not add
 // waits for memory to them: summing the ranges inside it, four steps at a time, took 8
 // aircraft, 90 steps, L 200, M 40 from 457 us (one kernel, checkpoints) to 1250 us, the
-// sums by a kernel of their own and the fetch ahead to 431 us.
+// sums by a kernel of their own and the fetch ahead to 429 us.
 #include "wind_rollout.cuh"
 
 #include <algorithm>
